@@ -46,6 +46,7 @@
 #include <vector>
 
 #include "ghb_internal.cuh"
+#include "passes_fx.cuh"
 
 namespace ghb {
 const char* last_error_cstr();
@@ -437,17 +438,27 @@ ghb_status prep_cg(ghb_batch* b, int op, std::vector<CgItem>& items, std::vector
 
 // Threads per CTA of a batched transform pass over `lines` interleaved lines
 // of length at most Mmax: about one thread per butterfly of a pass (a pass
-// combines up to 32 entries in FP32 and 18 in FP64, so a line has at least
-// Mmax / 32 or Mmax / 18 of them), in whole warps, at least 64.  Short
+// combines up to 32 entries, so a line has at least Mmax / 32 of them), in
+// whole warps, at least 64.  Short
 // transforms then run several CTAs per SM instead of one CTA whose threads
 // mostly wait.
 template <typename T>
 int batch_threads(int Mmax, int lines, int full) {
-  const int cap = sizeof(T) == 4 ? 32 : 18;
+  const int cap = 32;
   const int units = (Mmax + cap - 1) / cap;
   int t = ((units * lines + 31) / 32) * 32;
   if (t < 64) t = 64;
   return t < full ? t : full;
+}
+
+// FP64 passes over many operands: shared memory of `lines` lines of length at
+// most M (a line's padding is at most an eighth of it) and the columns per CTA
+// that leave room for several CTAs on an SM.
+size_t fx_smem_bound(int M, int lines) { return static_cast<size_t>(lines) * (M + M / 8) * sizeof(fx2); }
+int fx_batch_tile(int M) {
+  for (int tw : {8, 4, 2})
+    if (fx_smem_bound(M, tw) <= 56 * 1024) return tw;
+  return 1;
 }
 
 template <typename T>
@@ -461,11 +472,12 @@ ghb_status prep_col(ghb_batch* b, int sign, int mode, std::vector<ColItem>& item
   // autotuner's tile widths are timed on one operand and measured slower for
   // launches over many items of mixed lengths.  The items' radix groupings
   // (their plans) are the tuned ones.
-  const int TW = col_tile_width(Mmax, sizeof(C));
+  constexpr bool fx = sizeof(T) == 8;   // fixed-point passes: tiles of the flattened (outer, inner) range
+  const int TW = fx ? fx_batch_tile(Mmax) : col_tile_width(Mmax, sizeof(C));
   int64_t blocks = 0;
   for (auto& it : items) {
     it.block_begin = blocks;
-    blocks += ((it.a.inner + TW - 1) / TW) * it.a.outer;
+    blocks += fx ? (it.a.inner * it.a.outer + TW - 1) / TW : ((it.a.inner + TW - 1) / TW) * it.a.outer;
   }
   Launch L{};
   L.kind = 0;
@@ -473,10 +485,10 @@ ghb_status prep_col(ghb_batch* b, int sign, int mode, std::vector<ColItem>& item
   L.sign = sign;
   L.mode = mode;
   L.tile = TW;
-  L.threads = batch_threads<T>(Mmax, TW, sizeof(T) == 4 ? 512 : 256);
+  L.smem = fx ? fx_smem_bound(Mmax, TW) : col_smem_bytes(Mmax, TW, sizeof(C));
+  L.threads = fx ? fx_threads(Mmax, TW, Mmax + Mmax / 8) : batch_threads<T>(Mmax, TW, 512);
   L.n = static_cast<int>(items.size());
   L.blocks = blocks;
-  L.smem = col_smem_bytes(Mmax, TW, sizeof(C));
   const ColItem* dp = nullptr;
   TRYB(b->arena.push(items, &dp));
   L.items = dp;
@@ -506,10 +518,11 @@ ghb_status prep_row(ghb_batch* b, int mode, std::vector<RowItem>& items, const s
   L.f32 = sizeof(T) == 4;
   L.mode = mode;
   L.tile = NL;
-  L.threads = mode == ROW_MATVEC ? batch_threads<T>(Mmax, NL, 256) : 0;
+  constexpr bool fx = sizeof(T) == 8;
+  L.smem = fx ? fx_smem_bound(Mmax, NL) : padded_elems<C>(static_cast<size_t>(Mmax) * NL) * sizeof(C);
+  L.threads = fx ? fx_threads(Mmax, NL, Mmax + Mmax / 8) : (mode == ROW_MATVEC ? batch_threads<T>(Mmax, NL, 256) : 0);
   L.n = static_cast<int>(items.size());
   L.blocks = blocks;
-  L.smem = padded_elems<C>(static_cast<size_t>(Mmax) * NL) * sizeof(C);
   const RowItem* dp = nullptr;
   TRYB(b->arena.push(items, &dp));
   L.items = dp;

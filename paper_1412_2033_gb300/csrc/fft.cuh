@@ -83,24 +83,58 @@ enum PassShape {
   SH_COUNT
 };
 
+// Plan of the fixed-point FP64 transform (fft_fx.cuh).
+// w 2^62 of a root of unity: real part ch 2^32 + cl, imaginary part sh 2^32 +
+// sl, |cl|, |sl| < 2^31 (negation stays in range)
+struct alignas(16) fxw {
+  int ch, cl, sh, sl;
+};
+constexpr int kFxPasses = 12;
+enum FxShape { FX_2 = 0, FX_3, FX_4, FX_5, FX_3_2, FX_4_2, FX_3_3, FX_5_2, FX_GENERIC };
+
+// One pass of a plan.  Entry n of a line sits at position n + n / pad (pad = 0:
+// n): the first pass's butterflies read `pad` consecutive entries, and the
+// spare entry after each keeps neighbouring threads on different banks when
+// that count is even.  Later passes have strides that are multiples of pad.
+struct FxPass {
+  int shape;
+  int R;          // entries of one butterfly group
+  int lp;         // stride of the group in entries (product of the earlier passes)
+  int step;       // the same in positions
+  int block;      // lp R in positions
+  int units;      // groups per line
+  int ts;         // M / (lp R): twiddle step of the whole pass
+  int bits_dit, bits_dif;   // bits that the line's largest component may fill before the pass
+  FastDiv ulines;           // division by units
+  FastDiv ulp;              // division by lp
+};
+struct FxPlan {
+  int np;
+  int pad;        // 0 or the first pass's group size
+  int ls;         // positions of one line
+  FastDiv pdiv;   // division by pad (1 when pad = 0)
+  FxPass p[kFxPasses];
+  const int* perm;    // position of natural index n in digit-reversed order
+  const fxw* tw;      // tw[j] = exp(-2 pi i j / M) 2^62
+};
+
 // Plan of one length-M transform.  Tables live in device memory.
 struct FftPlan {
   int M;
   int nst;                   // number of stages
   int R[kMaxStages];         // radix of DIT stage t
   int Lp[kMaxStages];        // L_{t-1}: product of the radices before stage t
-  // passes per precision ([0] FP64: at most 18 entries per thread so the
-  // registers hold them; [1] FP32: at most 32)
-  int npass[2];
-  int pshape[2][kMaxPasses];    // PassShape of each pass (DIT order)
-  int pR[2][kMaxPasses];        // radix product of the pass (or the prime)
-  int pLp[2][kMaxPasses];       // L_{t-1} of its first stage
-  FastDiv pdiv[2][kMaxPasses];  // division by pLp
+  // passes of the FP32 transform (at most 32 entries per thread)
+  int npass;
+  int pshape[kMaxPasses];    // PassShape of each pass (DIT order)
+  int pR[kMaxPasses];        // radix product of the pass (or the prime)
+  int pLp[kMaxPasses];       // L_{t-1} of its first stage
+  FastDiv pdiv[kMaxPasses];  // division by pLp
   const int* perm;           // perm[n]: digit-reversed position of index n
   const int* perm_ct;        // the same for the stage order of fft_ct.cuh (null if M has no
                              // size-specialised kernels)
-  const double2* tw64;       // tw64[j] = exp(-2 pi i j / M)
-  const float2* tw32;        // the same rounded to float
+  const float2* tw32;        // tw32[j] = exp(-2 pi i j / M)
+  FxPlan fx;                 // the FP64 transform
   // launch configuration chosen by the autotuner (host-side choices; 0 = size rule)
   int tile[2];               // column-pass tile width ([0] FP64, [1] FP32)
   int rows32;                // rows per CTA of the FP32 2-D operator's last-axis pass
@@ -139,7 +173,6 @@ __device__ __forceinline__ C rot(C a) {
 }
 
 template <typename C> __device__ __forceinline__ const C* twtab(const FftPlan& p);
-template <> __device__ __forceinline__ const double2* twtab<double2>(const FftPlan& p) { return p.tw64; }
 template <> __device__ __forceinline__ const float2* twtab<float2>(const FftPlan& p) { return p.tw32; }
 
 // Padded shared-memory index: one spare slot every 128 bytes of data.
@@ -404,25 +437,16 @@ struct PassSmem {
 
 template <typename C>
 __device__ __forceinline__ int load_passes(PassSmem& s, const FftPlan& p) {
-  constexpr int k = sizeof(C) == 8 ? 1 : 0;
   if (threadIdx.x == 0) {
 #pragma unroll
     for (int i = 0; i < kMaxPasses; ++i) {
-      s.shape[i] = p.pshape[k][i];
-      s.R[i] = p.pR[k][i];
-      s.Lp[i] = p.pLp[k][i];
-      s.dv[i] = p.pdiv[k][i];
+      s.shape[i] = p.pshape[i];
+      s.R[i] = p.pR[i];
+      s.Lp[i] = p.pLp[i];
+      s.dv[i] = p.pdiv[i];
     }
   }
-  return p.npass[k];
-}
-
-// Passes wider than 18 entries run only in FP32 (the FP64 plans never use them,
-// and leaving them out keeps the FP64 kernels' register allocation small).
-template <int SIGN, bool DIT, int NL, int RA, int RB, int RC, typename C>
-__device__ __forceinline__ void run_pass_p(C* buf, int M, int Lp, const FastDiv& dv,
-                                           const C* __restrict__ tw) {
-  if constexpr (sizeof(C) == 8 || RA * RB * RC <= 18) run_pass<SIGN, DIT, NL, RA, RB, RC>(buf, M, Lp, dv, tw);
+  return p.npass;
 }
 
 template <int SIGN, bool DIT, int NL, typename C>
@@ -431,24 +455,24 @@ __device__ __forceinline__ void dispatch_pass(C* buf, int M, const PassSmem& ps,
   const int Lp = ps.Lp[i];
   const FastDiv dv = ps.dv[i];
   switch (ps.shape[i]) {
-    case SH_2: run_pass_p<SIGN, DIT, NL, 2, 1, 1>(buf, M, Lp, dv, tw); break;
-    case SH_3: run_pass_p<SIGN, DIT, NL, 3, 1, 1>(buf, M, Lp, dv, tw); break;
-    case SH_4: run_pass_p<SIGN, DIT, NL, 4, 1, 1>(buf, M, Lp, dv, tw); break;
-    case SH_5: run_pass_p<SIGN, DIT, NL, 5, 1, 1>(buf, M, Lp, dv, tw); break;
-    case SH_2_3: run_pass_p<SIGN, DIT, NL, 2, 3, 1>(buf, M, Lp, dv, tw); break;
-    case SH_3_3: run_pass_p<SIGN, DIT, NL, 3, 3, 1>(buf, M, Lp, dv, tw); break;
-    case SH_2_5: run_pass_p<SIGN, DIT, NL, 2, 5, 1>(buf, M, Lp, dv, tw); break;
-    case SH_4_3: run_pass_p<SIGN, DIT, NL, 4, 3, 1>(buf, M, Lp, dv, tw); break;
-    case SH_3_5: run_pass_p<SIGN, DIT, NL, 3, 5, 1>(buf, M, Lp, dv, tw); break;
-    case SH_4_4: run_pass_p<SIGN, DIT, NL, 4, 4, 1>(buf, M, Lp, dv, tw); break;
-    case SH_4_5: run_pass_p<SIGN, DIT, NL, 4, 5, 1>(buf, M, Lp, dv, tw); break;
-    case SH_5_5: run_pass_p<SIGN, DIT, NL, 5, 5, 1>(buf, M, Lp, dv, tw); break;
-    case SH_4_2: run_pass_p<SIGN, DIT, NL, 4, 2, 1>(buf, M, Lp, dv, tw); break;
-    case SH_2_3_3: run_pass_p<SIGN, DIT, NL, 2, 3, 3>(buf, M, Lp, dv, tw); break;
-    case SH_3_3_3: run_pass_p<SIGN, DIT, NL, 3, 3, 3>(buf, M, Lp, dv, tw); break;
-    case SH_4_2_3: run_pass_p<SIGN, DIT, NL, 4, 2, 3>(buf, M, Lp, dv, tw); break;
-    case SH_2_3_5: run_pass_p<SIGN, DIT, NL, 2, 3, 5>(buf, M, Lp, dv, tw); break;
-    case SH_4_4_2: run_pass_p<SIGN, DIT, NL, 4, 4, 2>(buf, M, Lp, dv, tw); break;
+    case SH_2: run_pass<SIGN, DIT, NL, 2, 1, 1>(buf, M, Lp, dv, tw); break;
+    case SH_3: run_pass<SIGN, DIT, NL, 3, 1, 1>(buf, M, Lp, dv, tw); break;
+    case SH_4: run_pass<SIGN, DIT, NL, 4, 1, 1>(buf, M, Lp, dv, tw); break;
+    case SH_5: run_pass<SIGN, DIT, NL, 5, 1, 1>(buf, M, Lp, dv, tw); break;
+    case SH_2_3: run_pass<SIGN, DIT, NL, 2, 3, 1>(buf, M, Lp, dv, tw); break;
+    case SH_3_3: run_pass<SIGN, DIT, NL, 3, 3, 1>(buf, M, Lp, dv, tw); break;
+    case SH_2_5: run_pass<SIGN, DIT, NL, 2, 5, 1>(buf, M, Lp, dv, tw); break;
+    case SH_4_3: run_pass<SIGN, DIT, NL, 4, 3, 1>(buf, M, Lp, dv, tw); break;
+    case SH_3_5: run_pass<SIGN, DIT, NL, 3, 5, 1>(buf, M, Lp, dv, tw); break;
+    case SH_4_4: run_pass<SIGN, DIT, NL, 4, 4, 1>(buf, M, Lp, dv, tw); break;
+    case SH_4_5: run_pass<SIGN, DIT, NL, 4, 5, 1>(buf, M, Lp, dv, tw); break;
+    case SH_5_5: run_pass<SIGN, DIT, NL, 5, 5, 1>(buf, M, Lp, dv, tw); break;
+    case SH_4_2: run_pass<SIGN, DIT, NL, 4, 2, 1>(buf, M, Lp, dv, tw); break;
+    case SH_2_3_3: run_pass<SIGN, DIT, NL, 2, 3, 3>(buf, M, Lp, dv, tw); break;
+    case SH_3_3_3: run_pass<SIGN, DIT, NL, 3, 3, 3>(buf, M, Lp, dv, tw); break;
+    case SH_4_2_3: run_pass<SIGN, DIT, NL, 4, 2, 3>(buf, M, Lp, dv, tw); break;
+    case SH_2_3_5: run_pass<SIGN, DIT, NL, 2, 3, 5>(buf, M, Lp, dv, tw); break;
+    case SH_4_4_2: run_pass<SIGN, DIT, NL, 4, 4, 2>(buf, M, Lp, dv, tw); break;
     default: run_generic<SIGN, DIT, NL>(buf, M, ps.R[i], Lp, dv, tw); break;
   }
 }

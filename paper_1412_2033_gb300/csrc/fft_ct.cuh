@@ -118,45 +118,10 @@ __device__ __forceinline__ void substage_const(C* v) {
   if constexpr (JP + 1 < SIG) substage_const<SIGN, DIT, RHO, SIG, RG, JP + 1>(v);
 }
 
-// One sub-stage with every twiddle read from the length-M table: entry offset
-// JP < SIG of the sub-stage takes (w_{L_s}^p w_{SIG RHO}^JP)^q = w_M^(q B),
-// B = TS p + JP M / (SIG RHO), for q = 1 .. RHO-1 (q B < M).  FP64 passes are
-// bound by the FP64 pipe, so table loads replace the complex products that
-// substage_jp spends on forming the powers (a fifth of their twiddle work).
-// FP32 passes keep substage_jp: they are bound by instruction issue and load
-// latency, and the table loads made the M = 4374 last-axis pass 145 -> 170 us.
-template <int SIGN, bool DIT, int RHO, int SIG, int RG, int JP, int TS, int M, typename C>
-__device__ __forceinline__ void substage_tab(C* v, int p, const C* __restrict__ tw) {
-  const int b = TS * p + JP * (M / (SIG * RHO));
-  C tq[RHO];
-#pragma unroll
-  for (int q = 1; q < RHO; ++q) tq[q] = __ldg(&tw[q * b]);
-#pragma unroll
-  for (int jb = 0; jb < RG / (SIG * RHO); ++jb) {
-    C e[RHO];
-#pragma unroll
-    for (int q = 0; q < RHO; ++q) e[q] = v[jb * SIG * RHO + JP + q * SIG];
-    if constexpr (DIT) {
-#pragma unroll
-      for (int q = 1; q < RHO; ++q) e[q] = twmul<SIGN>(e[q], tq[q]);
-    }
-    dft_small<SIGN, RHO>(e);
-    if constexpr (!DIT) {
-#pragma unroll
-      for (int q = 1; q < RHO; ++q) e[q] = twmul<SIGN>(e[q], tq[q]);
-    }
-#pragma unroll
-    for (int q = 0; q < RHO; ++q) v[jb * SIG * RHO + JP + q * SIG] = e[q];
-  }
-  if constexpr (JP + 1 < SIG) substage_tab<SIGN, DIT, RHO, SIG, RG, JP + 1, TS, M>(v, p, tw);
-}
-
 template <int SIGN, bool DIT, bool FIRST, int RHO, int SIG, int RG, int TS, int M, typename C>
 __device__ __forceinline__ void ct_substage(C* v, int p, const C* __restrict__ tw) {
   if constexpr (FIRST) {
     substage_const<SIGN, DIT, RHO, SIG, RG, 0>(v);
-  } else if constexpr (sizeof(C) == 16) {
-    substage_tab<SIGN, DIT, RHO, SIG, RG, 0, TS, M>(v, p, tw);
   } else {
     const C wb = __ldg(&tw[p * TS]);   // w_{L_s}^p
     substage_jp<SIGN, DIT, RHO, SIG, RG, 0>(v, wb);

@@ -109,26 +109,32 @@ struct PlanHolder {
   FftPlan plan{};
   int* d_perm = nullptr;
   int* d_perm_ct = nullptr;
-  double2* d_tw64 = nullptr;
   float2* d_tw32 = nullptr;
+  int* d_fx_perm = nullptr;   // digit reversal of the FP64 transform's current grouping
+  fxw* d_fx_tw = nullptr;
+  int fx_cap = 0;             // group-size cap of that grouping
 };
 
 // Plan with tables on the device and the autotuned launch configuration
 // (make_plan) or the size rules (make_plan_untuned).
 ghb_status make_plan(int M, PlanHolder& out);
 ghb_status make_plan_untuned(int M, PlanHolder& out);
-// Regroup the stages of precision k ([0] FP64, [1] FP32) into passes of radix
-// product <= maxprod.
-void group_passes(FftPlan& p, int k, int maxprod);
+// Regroup the stages of the FP32 transform into passes of radix product <= maxprod.
+void group_passes(FftPlan& p, int maxprod);
+// Regroup the FP64 transform into passes of group size <= cap (5 at least) and
+// replace its digit-reversal table on the device.
+constexpr int kFxCap = 18;
+ghb_status set_fx_cap(PlanHolder& h, int cap);
 // Write the autotuned configuration for length M into p (tuning M first if
 // it has not been tuned in this process and tuning is enabled).
-ghb_status apply_tune(int M, FftPlan& p);
+ghb_status apply_tune(int M, PlanHolder& h);
 // Host tables of a plan (digit reversal, twiddles); the
 // plan's device pointers are left null for the caller to place the tables.
 struct PlanTables {
   std::vector<int> perm;
-  std::vector<double2> tw64;
   std::vector<float2> tw32;
+  std::vector<int> fx_perm;
+  std::vector<fxw> fx_tw;
 };
 ghb_status build_plan_tables(int M, FftPlan& p, PlanTables& t);
 void free_plan(PlanHolder& p);

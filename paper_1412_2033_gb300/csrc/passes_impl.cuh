@@ -25,6 +25,7 @@
 
 #include "fft_ct.cuh"
 #include "ghb_internal.cuh"
+#include "launch_util.cuh"
 #include "reduce.cuh"
 
 namespace ghb {
@@ -46,22 +47,6 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 // wait until at most N of this thread's committed groups are still in flight
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
-
-// The dynamic shared-memory limit of kernel `func` raised to `bytes` on the
-// current device.  The attribute belongs to the device's context, so it is set
-// once per device (bit `dev` of `mask`, one mask per kernel); two host threads
-// may both set it, which is harmless.  Devices beyond 63 set it every time.
-template <typename F>
-inline ghb_status ensure_dyn_smem(F* func, int bytes, std::atomic<unsigned long long>& mask) {
-  int dev = 0;
-  GHB_CUDA_TRY(cudaGetDevice(&dev));
-  const unsigned long long bit = dev < 64 ? (1ull << dev) : 0ull;
-  if (bit == 0 || !(mask.load(std::memory_order_acquire) & bit)) {
-    GHB_CUDA_TRY(cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-    mask.fetch_or(bit, std::memory_order_release);
-  }
-  return GHB_OK;
-}
 
 // Shared-memory index of entry i: padded for the runtime-plan transform,
 // plain for the size-specialised one (MCT = its compile-time length).
@@ -353,18 +338,6 @@ template <typename T, int TW, int SIGN, int MODE, int MCT = 0>
 __global__ void __launch_bounds__(col_threads<T, TW, MCT, MODE>(), col_min_blocks<T, TW, MCT, MODE>())
     col_kernel(ColArgs a, FftPlan pl) {
   col_body<T, TW, SIGN, MODE, MCT>(a, pl, blockIdx.x);
-}
-
-// Index of the work item owning block `b` (items sorted by block_begin).
-template <typename Item>
-__device__ __forceinline__ int find_item(const Item* items, int n, int64_t b) {
-  int lo = 0, hi = n - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (items[mid].block_begin <= b) lo = mid;
-    else hi = mid - 1;
-  }
-  return lo;
 }
 
 // Many operands (instances, solves) in one launch: each item owns a

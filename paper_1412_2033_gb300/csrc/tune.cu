@@ -55,15 +55,20 @@ Tune size_rules(int M) {
   return Tune{32, 0, 0, ct, ct, 18, 0};
 }
 
-void write_tune(const Tune& t, FftPlan& p) {
-  group_passes(p, 1, t.cap32);
-  group_passes(p, 0, t.cap64);
+ghb_status write_tune(const Tune& t, PlanHolder& h) {
+  FftPlan& p = h.plan;
+  group_passes(p, t.cap32);
+  if (h.fx_cap != t.cap64) {
+    const ghb_status st = set_fx_cap(h, t.cap64);
+    if (st != GHB_OK) return st;
+  }
   p.tile[1] = t.tile32;
   p.tile[0] = t.tile64;
   p.rows32 = t.rows32;
   const bool ct = p.perm_ct != nullptr && ct_size(p.M);
   p.ct_col = ct ? t.ct_col : 0;
   p.ct_row = ct ? t.ct_row : 0;
+  return GHB_OK;
 }
 
 struct Timer {
@@ -155,7 +160,7 @@ ghb_status tune_length(int M, Tune* out) {
     TUNE_TRY(make_plan_untuned(M, fresh));
     plans[key] = fresh;
   }
-  const PlanHolder& ph = plans[key];
+  PlanHolder& ph = plans[key];
   Timer tm;
   TUNE_TRY(tm.init());
   struct {
@@ -211,7 +216,7 @@ ghb_status tune_length(int M, Tune* out) {
     float best_total = 1e30f, best_col_generic = 1e30f, best_row_generic = 1e30f;
     for (int cap : {18, 32}) {
       FftPlan p = ph.plan;
-      group_passes(p, 1, cap);
+      group_passes(p, cap);
       p.ct_col = p.ct_row = 0;
       float col_best = 1e30f, row_best = 1e30f;
       int rows_best = 0;
@@ -267,8 +272,8 @@ ghb_status tune_length(int M, Tune* out) {
     args(false, inv, fwd, row);
     float best_total = 1e30f;
     for (int cap : {9, 18}) {
+      TUNE_TRY(set_fx_cap(ph, cap));
       FftPlan p = ph.plan;
-      group_passes(p, 0, cap);
       float col_best = 1e30f;
       {
         p.tile[0] = 0;
@@ -324,12 +329,11 @@ ghb_status tune_of(int M, Tune* out) {
 
 namespace ghb {
 
-ghb_status apply_tune(int M, FftPlan& p) {
+ghb_status apply_tune(int M, PlanHolder& h) {
   Tune t{};
   const ghb_status st = tune_of(M, &t);
   if (st != GHB_OK) return st;
-  write_tune(t, p);
-  return GHB_OK;
+  return write_tune(t, h);
 }
 
 }  // namespace ghb

@@ -372,21 +372,22 @@ ghb_status ghb_gram_noalloc(int d, const int* N, const int* M, const double* gri
  * it decides how the FFTs of Algorithm 2 are laid out on the GPU, not what
  * they compute).  Per transform length M the library holds
  *   cfg[0] cap32   largest radix product of one register-blocked pass of the
- *                  runtime-plan FP32 transform (5..32)
- *   cfg[1] tile32  columns per CTA of the FP32 column passes (0 = chosen at
- *                  each launch from the operand's shape: the widest tile whose
- *                  CTAs fill the device three times over; else 1, 2, 4, 8 or 16
- *                  within shared memory, forced)
- *   cfg[2] rows32  rows per CTA of the FP32 2-D last-axis pass (0 = size rule,
- *                  1 or 2)
+ *                  runtime-plan FP32 transform (5..32; no pass is larger than
+ *                  16, so larger values are one setting)
+ *   cfg[1] tile32  columns per CTA of the runtime-plan FP32 column passes (0 =
+ *                  chosen at each launch from the operand's shape: the widest
+ *                  tile that leaves room for three CTAs on an SM and makes two
+ *                  for each; else 1, 2, 4, 8 or 16 within shared memory, forced)
+ *   cfg[2] rows32  rows per CTA of the FP32 2-D last-axis pass (0 = size rule;
+ *                  1 or 2: the least rows that fill complex lines, once or twice)
  *   cfg[3] ct_col  1: size-specialised FP32 column kernels (only for lengths
  *                  that have them: 72, 135, 162, 270, 486, 1458, 2187,
  *                  4374), 0: runtime plan
  *   cfg[4] ct_row  the same for the last-axis pass
- *   cfg[5] cap64   as cap32 for FP64
+ *   cfg[5] cap64   as cap32 for FP64 (no pass larger than 10)
  *   cfg[6] tile64  as tile32 for FP64
- * The first plan for M in a process times the candidates for cfg[0], [2], [3],
- * [4] and [5] on a 2-D operand of at least 2^20 double-grid entries with CUDA
+ * The first plan for M in a process times the candidates for cfg[2], [3], [4]
+ * and [5] on a 2-D operand of at least 2^20 double-grid entries with CUDA
  * events and keeps the fastest (the autotuner; the tiles stay 0); setting the
  * environment variable GHB_AUTOTUNE=0 keeps the size rules instead.  Every
  * configuration computes the same operator; results differ only by rounding.

@@ -17,7 +17,7 @@ CSRC = os.path.join(PKG, "csrc")
 LIBDIR = os.path.join(PKG, "lib")
 LIB = os.path.join(LIBDIR, "libghb.so")
 BUILD = os.path.join(ROOT, "_build")
-SOURCES = ["fx_row.cu", "fx_col.cu", "col_f32_a.cu", "col_f32_b.cu", "row_f32.cu",
+SOURCES = ["fx_row.cu", "fx_col.cu", "rt_row.cu", "rt_col.cu",
            "passes.cu", "plan.cu", "fields.cu", "api.cu", "batch.cu", "noalloc.cu",
            "ct_162.cu", "ct_486.cu", "ct_1458.cu", "ct_4374.cu", "ct_2187.cu",
            "ct_72.cu", "ct_135.cu", "ct_270.cu", "tune.cu"]

@@ -47,6 +47,7 @@
 
 #include "ghb_internal.cuh"
 #include "passes_fx.cuh"
+#include "passes_rt.cuh"
 
 namespace ghb {
 const char* last_error_cstr();
@@ -436,28 +437,22 @@ ghb_status prep_cg(ghb_batch* b, int op, std::vector<CgItem>& items, std::vector
   return GHB_OK;
 }
 
-// Threads per CTA of a batched transform pass over `lines` interleaved lines
-// of length at most Mmax: about one thread per butterfly of a pass (a pass
-// combines up to 32 entries, so a line has at least Mmax / 32 of them), in
-// whole warps, at least 64.  Short
-// transforms then run several CTAs per SM instead of one CTA whose threads
-// mostly wait.
+// Passes over many operands: the longest line of the launch (the plans' own line
+// lengths, which hold spare entries beyond M) and the lines per CTA that leave
+// room for several CTAs on an SM.
 template <typename T>
-int batch_threads(int Mmax, int lines, int full) {
-  const int cap = 32;
-  const int units = (Mmax + cap - 1) / cap;
-  int t = ((units * lines + 31) / 32) * 32;
-  if (t < 64) t = 64;
-  return t < full ? t : full;
+int longest_line(const ghb_batch* b, const std::vector<int>& Ms) {
+  int ls = 1;
+  for (int M : Ms) {
+    const FftPlan& p = b->plans.at(M).h.plan;
+    ls = std::max(ls, sizeof(T) == 8 ? p.fx.ls : p.rt.ls);
+  }
+  return ls;
 }
-
-// FP64 passes over many operands: shared memory of `lines` lines of length at
-// most M (a line's padding is at most an eighth of it) and the columns per CTA
-// that leave room for several CTAs on an SM.
-size_t fx_smem_bound(int M, int lines) { return static_cast<size_t>(lines) * (M + M / 8) * sizeof(fx2); }
-int fx_batch_tile(int M) {
-  for (int tw : {8, 4, 2})
-    if (fx_smem_bound(M, tw) <= 56 * 1024) return tw;
+template <typename T>
+int batch_lines(int ls) {
+  for (int n : {16, 8, 4, 2})
+    if (static_cast<size_t>(n) * ls * 2 * sizeof(T) <= 56 * 1024) return n;
   return 1;
 }
 
@@ -465,19 +460,20 @@ template <typename T>
 ghb_status prep_col(ghb_batch* b, int sign, int mode, std::vector<ColItem>& items, const std::vector<int>& Ms,
                     std::vector<Launch>& out) {
   if (items.empty()) return GHB_OK;
-  using C = typename CT<T>::type;
   int Mmax = 1;
   for (int M : Ms) Mmax = std::max(Mmax, M);
   // Launch shapes of the batched passes follow the size rules: the
   // autotuner's tile widths are timed on one operand and measured slower for
   // launches over many items of mixed lengths.  The items' radix groupings
   // (their plans) are the tuned ones.
-  constexpr bool fx = sizeof(T) == 8;   // fixed-point passes: tiles of the flattened (outer, inner) range
-  const int TW = fx ? fx_batch_tile(Mmax) : col_tile_width(Mmax, sizeof(C));
+  // tiles of the flattened (outer, inner) range
+  constexpr bool f64 = sizeof(T) == 8;
+  const int ls = longest_line<T>(b, Ms) + 15;   // column_stride of any item
+  const int TW = batch_lines<T>(ls);
   int64_t blocks = 0;
   for (auto& it : items) {
     it.block_begin = blocks;
-    blocks += fx ? (it.a.inner * it.a.outer + TW - 1) / TW : ((it.a.inner + TW - 1) / TW) * it.a.outer;
+    blocks += (it.a.inner * it.a.outer + TW - 1) / TW;
   }
   Launch L{};
   L.kind = 0;
@@ -485,8 +481,8 @@ ghb_status prep_col(ghb_batch* b, int sign, int mode, std::vector<ColItem>& item
   L.sign = sign;
   L.mode = mode;
   L.tile = TW;
-  L.smem = fx ? fx_smem_bound(Mmax, TW) : col_smem_bytes(Mmax, TW, sizeof(C));
-  L.threads = fx ? fx_threads(Mmax, TW, Mmax + Mmax / 8) : batch_threads<T>(Mmax, TW, 512);
+  L.smem = static_cast<size_t>(TW) * ls * 2 * sizeof(T);
+  L.threads = f64 ? fx_threads(Mmax, TW, ls) : rt_threads(Mmax, TW, ls);
   L.n = static_cast<int>(items.size());
   L.blocks = blocks;
   const ColItem* dp = nullptr;
@@ -500,11 +496,13 @@ template <typename T>
 ghb_status prep_row(ghb_batch* b, int mode, std::vector<RowItem>& items, const std::vector<int>& Ms, int nfields,
                     int ncomp, std::vector<Launch>& out) {
   if (items.empty()) return GHB_OK;
-  using C = typename CT<T>::type;
   int Mmax = 1;
   for (int M : Ms) Mmax = std::max(Mmax, M);
+  constexpr bool f64 = sizeof(T) == 8;
+  const int ls = longest_line<T>(b, Ms);
   int rpc = 1, NL = 1;
-  row_lines(mode, nfields, ncomp, Mmax, 0, &rpc, &NL);
+  if (f64) row_lines(mode, nfields, ncomp, Mmax, 0, &rpc, &NL);
+  else rt_row_shape(ncomp, Mmax, ls, 1 << 30, 0, &rpc, &NL);
   int64_t blocks = 0;
   for (auto& it : items) {
     it.rows_per_cta = rpc;
@@ -518,9 +516,8 @@ ghb_status prep_row(ghb_batch* b, int mode, std::vector<RowItem>& items, const s
   L.f32 = sizeof(T) == 4;
   L.mode = mode;
   L.tile = NL;
-  constexpr bool fx = sizeof(T) == 8;
-  L.smem = fx ? fx_smem_bound(Mmax, NL) : padded_elems<C>(static_cast<size_t>(Mmax) * NL) * sizeof(C);
-  L.threads = fx ? fx_threads(Mmax, NL, Mmax + Mmax / 8) : (mode == ROW_MATVEC ? batch_threads<T>(Mmax, NL, 256) : 0);
+  L.smem = static_cast<size_t>(NL) * ls * 2 * sizeof(T);
+  L.threads = f64 ? fx_threads(Mmax, NL, ls) : rt_threads(Mmax, NL, ls);
   L.n = static_cast<int>(items.size());
   L.blocks = blocks;
   const RowItem* dp = nullptr;

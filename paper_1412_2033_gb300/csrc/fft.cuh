@@ -9,10 +9,6 @@
 //     X[k] = sum_m u[m] exp(-2 pi i m k / M)          (SIGN = -1; the 1/M
 // factor is applied by the caller when it truncates to Z_N).
 //
-// Data layout in shared memory: NL independent lines interleaved,
-// element (m, line) at padded index pad(m * NL + line), so that consecutive
-// threads touch consecutive words and strided butterflies spread over banks.
-//
 // Algorithm (in place, one shared buffer).  M = R_1 ... R_s (radices 2,3,4,5 or
 // a prime <= 31).  Decimation in time (DIT) takes digit-reversed input (the
 // caller scatters x[n] to position perm[n]) and returns natural order; stage t
@@ -24,14 +20,17 @@
 // perm[k]).  A line therefore goes inverse (DIT) -> pointwise multiply ->
 // forward (DIF) without any permutation pass.
 //
-// Register blocking: consecutive stages are grouped into passes of at most
-// three stages (radix product <= 32).  The stages of a group act inside the
-// sets {b L_g + p + j L_{t-1} : j < R_g}, so one thread loads such a set into
-// registers, runs the group's stages there and writes it back: one shared-memory
-// round trip and one barrier per pass instead of per stage.  Twiddles: the
-// stage-s factor w_{L_s}^{(p + j' L_{t-1}) q} = (w_{L_s}^p w_{sigma rho}^{j'})^q is a
-// table load per pass and sub-stage (w_{L_s}^p) times a root of unity of small
-// order that the compiler evaluates, raised to the power q by multiplication.
+// Register blocking: consecutive stages are grouped into passes.  The stages of a
+// group act inside the sets {b L_g + p + j L_{t-1} : j < R_g}, so one thread
+// loads such a set into registers, runs the group's stages there and writes it
+// back: one shared-memory round trip and one barrier per pass instead of per
+// stage.  Twiddles: the stage-s factor w_{L_s}^{(p + j' L_{t-1}) q} = (w_{L_s}^p
+// w_{sigma rho}^{j'})^q is a table load per pass and sub-stage (w_{L_s}^p) times
+// a root of unity of small order that the compiler evaluates, raised to the
+// power q by multiplication.
+//
+// Three engines share the stages: fft_rt.cuh (FP32, plans known at run time),
+// fft_ct.cuh (FP32, lengths known at compile time) and fft_fx.cuh (FP64).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -40,7 +39,6 @@
 namespace ghb {
 
 constexpr int kMaxStages = 24;
-constexpr int kMaxPasses = 24;
 constexpr int kMaxGenericRadix = 31;
 
 // Division by an invariant 32-bit integer with a multiply-high (Granlund and
@@ -74,67 +72,70 @@ __device__ __forceinline__ unsigned fdiv(unsigned n, const FastDiv& f) {
   return (t + ((n - t) >> 1)) >> (f.l - 1);
 }
 
-// Shapes of one pass: the radices of its stages in DIT order.
-enum PassShape {
-  SH_2 = 0, SH_3, SH_4, SH_5,
-  SH_2_3, SH_3_3, SH_2_5, SH_4_3, SH_3_5, SH_4_4, SH_4_5, SH_5_5, SH_4_2,
-  SH_2_3_3, SH_3_3_3, SH_4_2_3, SH_2_3_5, SH_4_4_2,
-  SH_GENERIC,   // one stage of a prime radix 7..31 (O(R^2) definition)
-  SH_COUNT
-};
-
-// Plan of the fixed-point FP64 transform (fft_fx.cuh).
 // w 2^62 of a root of unity: real part ch 2^32 + cl, imaginary part sh 2^32 +
 // sl, |cl|, |sl| < 2^31 (negation stays in range)
 struct alignas(16) fxw {
   int ch, cl, sh, sl;
 };
+
+// Run-time plans of the transforms: FP64 in fixed point (fft_fx.cuh) and FP32
+// (fft_rt.cuh).
 constexpr int kFxPasses = 12;
 enum FxShape { FX_2 = 0, FX_3, FX_4, FX_5, FX_3_2, FX_4_2, FX_3_3, FX_5_2, FX_GENERIC };
+enum RtShape {
+  RT_2 = 0, RT_3, RT_4, RT_5, RT_3_2, RT_4_2, RT_3_3, RT_5_2, RT_GENERIC, RT_3_4, RT_5_3, RT_4_4
+};
 
-// One pass of a plan.  Entry n of a line sits at position n + n / pad (pad = 0:
-// n): the first pass's butterflies read `pad` consecutive entries, and the
-// spare entry after each keeps neighbouring threads on different banks when
-// that count is even.  Later passes have strides that are multiples of pad.
+// One pass.  Entry i of a line sits at position nat[i] = i plus one spare entry
+// for every completed block of the passes whose block length in positions would
+// be a multiple of 4 (neighbouring threads would share banks); inside a group
+// the positions are evenly spaced (step).
 struct FxPass {
-  int shape;
+  int shape;      // FxShape or RtShape (the common ones have the same numbers)
   int R;          // entries of one butterfly group
   int lp;         // stride of the group in entries (product of the earlier passes)
   int step;       // the same in positions
-  int block;      // lp R in positions
   int units;      // groups per line
   int ts;         // M / (lp R): twiddle step of the whole pass
-  int bits_dit, bits_dif;   // bits that the line's largest component may fill before the pass
+  int bits_dit, bits_dif;   // FP64: bits that the line's largest component may fill before the pass
   FastDiv ulines;           // division by units
   FastDiv ulp;              // division by lp
 };
 struct FxPlan {
+  int M;
   int np;
-  int pad;        // 0 or the first pass's group size
-  int ls;         // positions of one line
-  FastDiv pdiv;   // division by pad (1 when pad = 0)
+  int ls;              // positions of one line
+  const int* perm;     // position of natural index n in digit-reversed order
+  const int* nat;      // position of entry i
+  const fxw* tw;       // FP64: tw[j] = exp(-2 pi i j / M) 2^62
+  const float2* tw32;  // FP32: tw32[j] = exp(-2 pi i j / M)
   FxPass p[kFxPasses];
-  const int* perm;    // position of natural index n in digit-reversed order
-  const fxw* tw;      // tw[j] = exp(-2 pi i j / M) 2^62
 };
 
-// Plan of one length-M transform.  Tables live in device memory.
+// Distance of the TW (a power of two, <= 16) lines of a column tile, whose
+// neighbouring threads alternate between lines: ls or up to 15 more, = 16 / TW
+// modulo 16 entries of 8 bytes (8 / TW modulo 8 of 16 bytes), so that the lines' threads
+// and the neighbouring entries of each line share no bank.
+__host__ __device__ inline int column_stride(int ls, int TW, int entry_bytes) {
+  const int period = 128 / entry_bytes;
+  const int want = TW < period ? period / TW : 1;
+  return ls + ((want - ls) & (period - 1));
+}
+
+// Tables of the size-specialised kernels: the digit-reversed position of natural
+// index n in the stage order of fft_ct.cuh, and the roots tw[j] = exp(-2 pi i j / M).
+struct CtTables {
+  const int* perm;
+  const float2* tw;
+};
+
+// Plan of one length-M transform.  Tables live in device memory.  A kernel takes
+// the part that it runs on, not the whole: a launch writes its arguments out.
 struct FftPlan {
   int M;
-  int nst;                   // number of stages
-  int R[kMaxStages];         // radix of DIT stage t
-  int Lp[kMaxStages];        // L_{t-1}: product of the radices before stage t
-  // passes of the FP32 transform (at most 32 entries per thread)
-  int npass;
-  int pshape[kMaxPasses];    // PassShape of each pass (DIT order)
-  int pR[kMaxPasses];        // radix product of the pass (or the prime)
-  int pLp[kMaxPasses];       // L_{t-1} of its first stage
-  FastDiv pdiv[kMaxPasses];  // division by pLp
-  const int* perm;           // perm[n]: digit-reversed position of index n
-  const int* perm_ct;        // the same for the stage order of fft_ct.cuh (null if M has no
-                             // size-specialised kernels)
-  const float2* tw32;        // tw32[j] = exp(-2 pi i j / M)
+  CtTables ct;               // null if M has no size-specialised kernels
   FxPlan fx;                 // the FP64 transform
+  FxPlan rt;                 // the FP32 transform
   // launch configuration chosen by the autotuner (host-side choices; 0 = size rule)
   int tile[2];               // column-pass tile width ([0] FP64, [1] FP32)
   int rows32;                // rows per CTA of the FP32 2-D operator's last-axis pass
@@ -172,14 +173,8 @@ __device__ __forceinline__ C rot(C a) {
   return SIGN > 0 ? mk(-a.y, a.x) : mk(a.y, -a.x);
 }
 
-template <typename C> __device__ __forceinline__ const C* twtab(const FftPlan& p);
-template <> __device__ __forceinline__ const float2* twtab<float2>(const FftPlan& p) { return p.tw32; }
-
-// Padded shared-memory index: one spare slot every 128 bytes of data.
-template <typename C>
-__device__ __forceinline__ int pidx(int i) {
-  return sizeof(C) == 8 ? i + (i >> 4) : i + (i >> 3);
-}
+// Entries of n with one spare every 128 bytes (the sizes that the launches admit
+// are stated in these terms).
 template <typename C>
 __host__ __device__ constexpr size_t padded_elems(size_t n) {
   return sizeof(C) == 8 ? n + (n >> 4) + 1 : n + (n >> 3) + 1;
@@ -341,159 +336,6 @@ __device__ __forceinline__ void substage_jp(C* v, C wb) {
     for (int q = 0; q < RHO; ++q) v[jb * SIG * RHO + JP + q * SIG] = e[q];
   }
   if constexpr (JP + 1 < SIG) substage_jp<SIGN, DIT, RHO, SIG, RG, JP + 1>(v, wb);
-}
-
-// One sub-stage of a register-blocked pass.  RHO: radix of the stage, SIG:
-// product of the radices before it inside the pass, RG: radix product of the
-// whole pass; v holds the pass's RG entries (entry j at position
-// b L_g + p + j Lp).  ts = M / (Lp SIG RHO).  The sub-stage's twiddle for
-// entry offset jp < SIG is w_{L_s}^p times the compile-time root w_{SIG RHO}^jp.
-template <int SIGN, bool DIT, int RHO, int SIG, int RG, typename C>
-__device__ __forceinline__ void substage(C* v, int p, int ts, const C* __restrict__ tw) {
-  const C wb = __ldg(&tw[p * ts]);   // w_{L_s}^p, L_s = Lp SIG RHO
-  substage_jp<SIGN, DIT, RHO, SIG, RG, 0>(v, wb);
-}
-
-// A pass of up to three stages (radices RA, RB, RC in DIT order; 1 = absent).
-template <int SIGN, bool DIT, int NL, int RA, int RB, int RC, typename C>
-__device__ __forceinline__ void run_pass(C* buf, int M, int Lp, const FastDiv& dv,
-                                         const C* __restrict__ tw) {
-  constexpr int RG = RA * RB * RC;
-  const int units = M / RG;
-  const int tsA = M / (Lp * RA);
-  const int tsB = tsA / RB;
-  const int tsC = tsB / RC;
-  for (int u = threadIdx.x; u < units * NL; u += blockDim.x) {
-    const int line = (NL == 1) ? 0 : u % NL;
-    const int unit = (NL == 1) ? u : u / NL;
-    const int b = static_cast<int>(fdiv(static_cast<unsigned>(unit), dv));
-    const int p = unit - b * Lp;
-    const int base = (b * Lp * RG + p) * NL + line;
-    const int step = Lp * NL;
-    C v[RG];
-#pragma unroll
-    for (int j = 0; j < RG; ++j) v[j] = buf[pidx<C>(base + j * step)];
-    if (DIT) {
-      substage<SIGN, DIT, RA, 1, RG>(v, p, tsA, tw);
-      if constexpr (RB > 1) substage<SIGN, DIT, RB, RA, RG>(v, p, tsB, tw);
-      if constexpr (RC > 1) substage<SIGN, DIT, RC, RA * RB, RG>(v, p, tsC, tw);
-    } else {
-      if constexpr (RC > 1) substage<SIGN, DIT, RC, RA * RB, RG>(v, p, tsC, tw);
-      if constexpr (RB > 1) substage<SIGN, DIT, RB, RA, RG>(v, p, tsB, tw);
-      substage<SIGN, DIT, RA, 1, RG>(v, p, tsA, tw);
-    }
-#pragma unroll
-    for (int j = 0; j < RG; ++j) buf[pidx<C>(base + j * step)] = v[j];
-  }
-}
-
-// One stage of a prime radix R <= kMaxGenericRadix by the O(R^2) definition,
-// with the R-th roots of unity taken from the length-M table (R divides M).
-template <int SIGN, bool DIT, int NL, typename C>
-__device__ void run_generic(C* buf, int M, int R, int Lp, const FastDiv& dv, const C* __restrict__ tw) {
-  const int units = M / R;
-  const int Lt = Lp * R;
-  const int ts = M / Lt;
-  const int MR = M / R;
-  for (int u = threadIdx.x; u < units * NL; u += blockDim.x) {
-    const int line = (NL == 1) ? 0 : u % NL;
-    const int unit = (NL == 1) ? u : u / NL;
-    const int b = static_cast<int>(fdiv(static_cast<unsigned>(unit), dv));
-    const int p = unit - b * Lp;
-    const int base = (b * Lt + p) * NL + line;
-    const int step = Lp * NL;
-    C v[kMaxGenericRadix];
-    C o[kMaxGenericRadix];
-    for (int q = 0; q < R; ++q) {
-      v[q] = buf[pidx<C>(base + q * step)];
-      if (DIT && q > 0) v[q] = twmul<SIGN>(v[q], __ldg(&tw[q * p * ts]));
-    }
-    for (int k = 0; k < R; ++k) {
-      C acc = v[0];
-      int e = 0;
-      for (int n = 1; n < R; ++n) {
-        e += k;
-        if (e >= R) e -= R;
-        acc = acc + twmul<SIGN>(v[n], __ldg(&tw[e * MR]));
-      }
-      o[k] = acc;
-    }
-    for (int q = 0; q < R; ++q) {
-      C r = o[q];
-      if (!DIT && q > 0) r = twmul<SIGN>(r, __ldg(&tw[q * p * ts]));
-      buf[pidx<C>(base + q * step)] = r;
-    }
-  }
-}
-
-// Pass metadata copied to shared memory once per kernel (avoids dynamic
-// indexing of kernel-parameter arrays).
-struct PassSmem {
-  int shape[kMaxPasses];
-  int R[kMaxPasses];
-  int Lp[kMaxPasses];
-  FastDiv dv[kMaxPasses];
-};
-
-template <typename C>
-__device__ __forceinline__ int load_passes(PassSmem& s, const FftPlan& p) {
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int i = 0; i < kMaxPasses; ++i) {
-      s.shape[i] = p.pshape[i];
-      s.R[i] = p.pR[i];
-      s.Lp[i] = p.pLp[i];
-      s.dv[i] = p.pdiv[i];
-    }
-  }
-  return p.npass;
-}
-
-template <int SIGN, bool DIT, int NL, typename C>
-__device__ __forceinline__ void dispatch_pass(C* buf, int M, const PassSmem& ps, int i,
-                                              const C* __restrict__ tw) {
-  const int Lp = ps.Lp[i];
-  const FastDiv dv = ps.dv[i];
-  switch (ps.shape[i]) {
-    case SH_2: run_pass<SIGN, DIT, NL, 2, 1, 1>(buf, M, Lp, dv, tw); break;
-    case SH_3: run_pass<SIGN, DIT, NL, 3, 1, 1>(buf, M, Lp, dv, tw); break;
-    case SH_4: run_pass<SIGN, DIT, NL, 4, 1, 1>(buf, M, Lp, dv, tw); break;
-    case SH_5: run_pass<SIGN, DIT, NL, 5, 1, 1>(buf, M, Lp, dv, tw); break;
-    case SH_2_3: run_pass<SIGN, DIT, NL, 2, 3, 1>(buf, M, Lp, dv, tw); break;
-    case SH_3_3: run_pass<SIGN, DIT, NL, 3, 3, 1>(buf, M, Lp, dv, tw); break;
-    case SH_2_5: run_pass<SIGN, DIT, NL, 2, 5, 1>(buf, M, Lp, dv, tw); break;
-    case SH_4_3: run_pass<SIGN, DIT, NL, 4, 3, 1>(buf, M, Lp, dv, tw); break;
-    case SH_3_5: run_pass<SIGN, DIT, NL, 3, 5, 1>(buf, M, Lp, dv, tw); break;
-    case SH_4_4: run_pass<SIGN, DIT, NL, 4, 4, 1>(buf, M, Lp, dv, tw); break;
-    case SH_4_5: run_pass<SIGN, DIT, NL, 4, 5, 1>(buf, M, Lp, dv, tw); break;
-    case SH_5_5: run_pass<SIGN, DIT, NL, 5, 5, 1>(buf, M, Lp, dv, tw); break;
-    case SH_4_2: run_pass<SIGN, DIT, NL, 4, 2, 1>(buf, M, Lp, dv, tw); break;
-    case SH_2_3_3: run_pass<SIGN, DIT, NL, 2, 3, 3>(buf, M, Lp, dv, tw); break;
-    case SH_3_3_3: run_pass<SIGN, DIT, NL, 3, 3, 3>(buf, M, Lp, dv, tw); break;
-    case SH_4_2_3: run_pass<SIGN, DIT, NL, 4, 2, 3>(buf, M, Lp, dv, tw); break;
-    case SH_2_3_5: run_pass<SIGN, DIT, NL, 2, 3, 5>(buf, M, Lp, dv, tw); break;
-    case SH_4_4_2: run_pass<SIGN, DIT, NL, 4, 4, 2>(buf, M, Lp, dv, tw); break;
-    default: run_generic<SIGN, DIT, NL>(buf, M, ps.R[i], Lp, dv, tw); break;
-  }
-}
-
-// Decimation in time: digit-reversed input -> natural output.  The caller
-// must __syncthreads() after filling buf; returns after a final barrier.
-template <int SIGN, int NL, typename C>
-__device__ void fft_dit(C* buf, const PassSmem& ps, int npass, int M, const C* tw) {
-  for (int i = 0; i < npass; ++i) {
-    dispatch_pass<SIGN, true, NL>(buf, M, ps, i, tw);
-    __syncthreads();
-  }
-}
-
-// Decimation in frequency: natural input -> digit-reversed output.
-template <int SIGN, int NL, typename C>
-__device__ void fft_dif(C* buf, const PassSmem& ps, int npass, int M, const C* tw) {
-  for (int i = npass - 1; i >= 0; --i) {
-    dispatch_pass<SIGN, false, NL>(buf, M, ps, i, tw);
-    __syncthreads();
-  }
 }
 
 }  // namespace ghb

@@ -64,7 +64,7 @@ FX_HD long long fx_wide(int a, int b, long long c) {
 }
 constexpr long long kFxHalf = 1LL << 31;
 
-// a + v C / 2^64, C = ch 2^32 + cl (|C| <= 2^62, |v| <= 2^62), error below one unit
+// a + v C / 2^64, C = ch 2^32 + cl (|C| <= 2^62, |v| < 2^63), error below one unit
 FX_HD long long fx_mul_add(long long v, int ch, int cl, long long a) {
   const int vl = static_cast<int>(v), vh = fx_hi(v);
   const long long cross = fx_wide(vh, cl, fx_wide(vl, ch, kFxHalf));
@@ -72,8 +72,9 @@ FX_HD long long fx_mul_add(long long v, int ch, int cl, long long a) {
 }
 
 // a w / 4 (SIGN = -1) or a conj(w) / 4 (SIGN = +1), w in the forward
-// convention, |components of a| <= 2^62 (the cross sums stay below 2^63 since
-// |ch| + |sh| <= sqrt(2) 2^30).
+// convention, |a| <= 2^62.8 (the cross sums stay below 2^63: |ch| + |sh| <=
+// sqrt(2) 2^30 against the low halves, |ah| + |bh| <= sqrt(2) |a| 2^-32 against
+// the roots' low halves).
 template <int SIGN>
 FX_HD fx2 fx_cmul4(fx2 a, fxw w) {
   const int sh = SIGN < 0 ? w.sh : -w.sh, sl = SIGN < 0 ? w.sl : -w.sl;
@@ -292,12 +293,13 @@ FX_HD int fx_tracked(int lo, int hi) { return hi > ~lo ? hi : ~lo; }   // lo <= 
 // ---------------------------------------------------------------------------
 // passes
 // ---------------------------------------------------------------------------
-// Host side (plan.cu): the passes of length M with group sizes <= cap, the
+// Host side (plan.cu): the passes (k = 0: these, 1: fft_rt.cuh's) of length M with group sizes <= cap, the
 // roots of unity and their fixed-point table.
 struct UnitRoot {
   long double c, s;   // cos, sin of 2 pi j / M
 };
-bool fx_group_passes(int M, int cap, FxPlan& f, std::vector<int>* perm_out);
+// (perm_out, nat_out: the tables of FxPlan, left out when null)
+bool group_plan(int k, int M, int cap, FxPlan& f, std::vector<int>* perm_out, std::vector<int>* nat_out);
 void unit_roots(int M, std::vector<UnitRoot>& r);
 void fx_twiddles(const std::vector<UnitRoot>& roots, std::vector<fxw>& tw);
 
@@ -444,23 +446,15 @@ FX_HD int fx_group_generic(fx2* base, int step, int g, int p, int R, int ts, int
   return fx_tracked(lo, hi);
 }
 
-// Unit u of a pass over one line: its first position and its offset p < lp.
-FX_HD int fx_unit_base(const FxPass& P, int pad, const FastDiv& pdiv, int u, int& p) {
+// First entry of unit u of a pass and its offset p < lp.
+FX_HD int fx_unit_entry(const FxPass& P, int u, int& p) {
 #ifdef __CUDA_ARCH__
   const int b = static_cast<int>(fdiv(static_cast<unsigned>(u), P.ulp));
 #else
   const int b = u / P.lp;
 #endif
   p = u - b * P.lp;
-  int pos = b * P.block + p;
-  if (pad > 0) {
-#ifdef __CUDA_ARCH__
-    pos += static_cast<int>(fdiv(static_cast<unsigned>(p), pdiv));
-#else
-    pos += p / pad;
-#endif
-  }
-  return pos;
+  return b * (P.lp * P.R) + p;
 }
 
 template <int SIGN, bool DIT, bool FIRST>

@@ -6,8 +6,8 @@ namespace ghb {
 
 template <int SIGN>
 __global__ void __launch_bounds__(kFxThreads, kFxBlocks)
-    fx_col_kernel(const __grid_constant__ ColArgs a, const __grid_constant__ FftPlan pl, int TW) {
-  fx_col_body<SIGN>(a, pl, TW, blockIdx.x);
+    fx_col_kernel(const __grid_constant__ ColArgs a, const __grid_constant__ FxPlan f, int TW) {
+  fx_col_body<SIGN>(a, f, TW, blockIdx.x);
 }
 
 template <int SIGN>
@@ -16,18 +16,18 @@ __global__ void __launch_bounds__(kFxThreads, kFxBlocks) fx_col_kernel_batch(con
   if (threadIdx.x == 0) s_item = find_item(items, n, blockIdx.x);
   __syncthreads();
   const ColItem& it = items[s_item];
-  fx_col_body<SIGN>(it.a, *it.pl, TW, blockIdx.x - it.block_begin);
+  fx_col_body<SIGN>(it.a, it.pl->fx, TW, blockIdx.x - it.block_begin);
 }
 
 namespace {
 
 template <int SIGN>
-ghb_status col_launch(const ColArgs& a, const FftPlan& pl, int TW, cudaStream_t s) {
+ghb_status col_launch(const ColArgs& a, const FxPlan& f, int TW, cudaStream_t s) {
   static std::atomic<unsigned long long> mask{0};
   TRY_STATUS(ensure_dyn_smem(fx_col_kernel<SIGN>, 220 * 1024, mask));
-  const size_t smem = static_cast<size_t>(TW) * pl.fx.ls * sizeof(fx2);
+  const size_t smem = static_cast<size_t>(TW) * column_stride(f.ls, TW, sizeof(fx2)) * sizeof(fx2);
   const int64_t grid = (a.outer * a.inner + TW - 1) / TW;
-  fx_col_kernel<SIGN><<<static_cast<unsigned>(grid), fx_threads(pl.M, TW, pl.fx.ls), smem, s>>>(a, pl, TW);
+  fx_col_kernel<SIGN><<<static_cast<unsigned>(grid), fx_threads(f.M, TW, f.ls), smem, s>>>(a, f, TW);
   GHB_CUDA_TRY(cudaGetLastError());
   return GHB_OK;
 }
@@ -44,8 +44,8 @@ ghb_status col_launch_batch(int TW, const ColItem* items, int n, int64_t blocks,
 
 }  // namespace
 
-ghb_status launch_fx_col(int sign, const ColArgs& a, const FftPlan& pl, int TW, cudaStream_t s) {
-  return sign > 0 ? col_launch<+1>(a, pl, TW, s) : col_launch<-1>(a, pl, TW, s);
+ghb_status launch_fx_col(int sign, const ColArgs& a, const FxPlan& f, int TW, cudaStream_t s) {
+  return sign > 0 ? col_launch<+1>(a, f, TW, s) : col_launch<-1>(a, f, TW, s);
 }
 
 ghb_status launch_fx_col_batch(int sign, int TW, const ColItem* items, int n, int64_t blocks, size_t smem, int threads,

@@ -6,8 +6,8 @@ namespace ghb {
 
 template <int MODE>
 __global__ void __launch_bounds__(kFxThreads, kFxBlocks)
-    fx_row_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ FftPlan pl, int rows_per_cta, int NL) {
-  fx_row_body<MODE>(a, pl, rows_per_cta, NL, blockIdx.x, gridDim.x);
+    fx_row_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ FxPlan f, int rows_per_cta, int NL) {
+  fx_row_body<MODE>(a, f, rows_per_cta, NL, blockIdx.x, gridDim.x);
 }
 
 template <int MODE>
@@ -16,19 +16,19 @@ __global__ void __launch_bounds__(kFxThreads, kFxBlocks) fx_row_kernel_batch(con
   if (threadIdx.x == 0) s_item = find_item(items, n, blockIdx.x);
   __syncthreads();
   const RowItem& it = items[s_item];
-  fx_row_body<MODE>(it.a, *it.pl, it.rows_per_cta, NL, blockIdx.x - it.block_begin, it.nblocks);
+  fx_row_body<MODE>(it.a, it.pl->fx, it.rows_per_cta, NL, blockIdx.x - it.block_begin, it.nblocks);
 }
 
 namespace {
 
 template <int MODE>
-ghb_status row_launch(const RowArgs& a, const FftPlan& pl, int rows_per_cta, int NL, int threads, cudaStream_t s) {
+ghb_status row_launch(const RowArgs& a, const FxPlan& f, int rows_per_cta, int NL, int threads, cudaStream_t s) {
   static std::atomic<unsigned long long> mask{0};
   TRY_STATUS(ensure_dyn_smem(fx_row_kernel<MODE>, 220 * 1024, mask));
-  const size_t smem = static_cast<size_t>(NL) * pl.fx.ls * sizeof(fx2);
+  const size_t smem = static_cast<size_t>(NL) * f.ls * sizeof(fx2);
   int64_t grid = (a.rows + rows_per_cta - 1) / rows_per_cta;
   if (MODE == ROW_ENERGY && grid > 1024) grid = 1024;   // partials hold 1024 x 6 doubles
-  fx_row_kernel<MODE><<<static_cast<unsigned>(grid), threads, smem, s>>>(a, pl, rows_per_cta, NL);
+  fx_row_kernel<MODE><<<static_cast<unsigned>(grid), threads, smem, s>>>(a, f, rows_per_cta, NL);
   GHB_CUDA_TRY(cudaGetLastError());
   return GHB_OK;
 }
@@ -45,12 +45,12 @@ ghb_status row_launch_batch(int NL, const RowItem* items, int n, int64_t blocks,
 
 }  // namespace
 
-ghb_status launch_fx_row(int mode, const RowArgs& a, const FftPlan& pl, int rows_per_cta, int NL, int threads,
+ghb_status launch_fx_row(int mode, const RowArgs& a, const FxPlan& f, int rows_per_cta, int NL, int threads,
                          cudaStream_t s) {
   switch (mode) {
-    case ROW_MATVEC: return row_launch<ROW_MATVEC>(a, pl, rows_per_cta, NL, threads, s);
-    case ROW_TOREAL: return row_launch<ROW_TOREAL>(a, pl, rows_per_cta, NL, threads, s);
-    default: return row_launch<ROW_ENERGY>(a, pl, rows_per_cta, NL, threads, s);
+    case ROW_MATVEC: return row_launch<ROW_MATVEC>(a, f, rows_per_cta, NL, threads, s);
+    case ROW_TOREAL: return row_launch<ROW_TOREAL>(a, f, rows_per_cta, NL, threads, s);
+    default: return row_launch<ROW_ENERGY>(a, f, rows_per_cta, NL, threads, s);
   }
 }
 

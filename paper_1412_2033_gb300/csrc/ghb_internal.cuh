@@ -107,33 +107,31 @@ struct Geometry {
 // Host-owned plan with its device tables.
 struct PlanHolder {
   FftPlan plan{};
-  int* d_perm = nullptr;
   int* d_perm_ct = nullptr;
   float2* d_tw32 = nullptr;
-  int* d_fx_perm = nullptr;   // digit reversal of the FP64 transform's current grouping
   fxw* d_fx_tw = nullptr;
-  int fx_cap = 0;             // group-size cap of that grouping
+  // digit reversal and positions (perm, then nat) and group-size cap of the
+  // transforms' current groupings ([0] FP64, [1] FP32)
+  int* d_group_perm[2] = {nullptr, nullptr};
+  int cap[2] = {0, 0};
 };
 
 // Plan with tables on the device and the autotuned launch configuration
 // (make_plan) or the size rules (make_plan_untuned).
 ghb_status make_plan(int M, PlanHolder& out);
 ghb_status make_plan_untuned(int M, PlanHolder& out);
-// Regroup the stages of the FP32 transform into passes of radix product <= maxprod.
-void group_passes(FftPlan& p, int maxprod);
-// Regroup the FP64 transform into passes of group size <= cap (5 at least) and
-// replace its digit-reversal table on the device.
-constexpr int kFxCap = 18;
-ghb_status set_fx_cap(PlanHolder& h, int cap);
+// Regroup the transform of precision k ([0] FP64, [1] FP32) into passes of group
+// size <= cap (5 at least) and replace its digit-reversal table on the device.
+constexpr int kGroupCap[2] = {18, 32};
+ghb_status set_group_cap(PlanHolder& h, int k, int cap);
 // Write the autotuned configuration for length M into p (tuning M first if
 // it has not been tuned in this process and tuning is enabled).
 ghb_status apply_tune(int M, PlanHolder& h);
 // Host tables of a plan (digit reversal, twiddles); the
 // plan's device pointers are left null for the caller to place the tables.
 struct PlanTables {
-  std::vector<int> perm;
   std::vector<float2> tw32;
-  std::vector<int> fx_perm;
+  std::vector<int> perm_of[2], nat_of[2];   // of the groupings, [0] FP64, [1] FP32
   std::vector<fxw> fx_tw;
 };
 ghb_status build_plan_tables(int M, FftPlan& p, PlanTables& t);
@@ -164,6 +162,10 @@ struct ColArgs {
 
 template <typename T>
 ghb_status launch_col(int sign, int mode, const ColArgs& a, const FftPlan& pl, cudaStream_t s);
+template <>
+ghb_status launch_col<float>(int sign, int mode, const ColArgs& a, const FftPlan& pl, cudaStream_t s);
+template <>
+ghb_status launch_col<double>(int sign, int mode, const ColArgs& a, const FftPlan& pl, cudaStream_t s);
 
 enum RowMode { ROW_MATVEC = 0, ROW_TOREAL = 1, ROW_ENERGY = 2 };
 
@@ -186,6 +188,10 @@ struct RowArgs {
 
 template <typename T>
 ghb_status launch_row(int mode, const RowArgs& a, const FftPlan& pl, cudaStream_t s);
+template <>
+ghb_status launch_row<float>(int mode, const RowArgs& a, const FftPlan& pl, cudaStream_t s);
+template <>
+ghb_status launch_row<double>(int mode, const RowArgs& a, const FftPlan& pl, cudaStream_t s);
 
 // Work items of batched launches: every item is one operand (an instance's
 // solve) with its own sizes and plan; it owns blocks [block_begin, block_begin + nblocks).
@@ -350,16 +356,14 @@ __host__ __device__ constexpr int col_tile_width(int M, int elem_bytes) {
   return 1;
 }
 
-// Transform lengths with size-specialised FP32 and FP64 operator kernels
+// Transform lengths with size-specialised FP32 operator kernels
 // (fft_ct.cuh): the double grids 2 * 3^k of the 2-D operator at N = 81, 243,
 // 729, 2187, 2187 itself (the reduced operator's transforms at N = 2187), and
 // the double grids 72, 135, 270 of the 3-D operator at N = 33, 65, 129.
 __host__ __device__ constexpr bool ct_size(int M) {
   return M == 162 || M == 486 || M == 1458 || M == 4374 || M == 2187 || M == 72 || M == 135 || M == 270;
 }
-template <typename T>
 ghb_status launch_col_ct(int sign, int mode, const ColArgs& a, const FftPlan& pl, cudaStream_t s);
-template <typename T>
 ghb_status launch_row_ct(int NL, const RowArgs& a, const FftPlan& pl, int rows_per_cta, cudaStream_t s);
 
 }  // namespace ghb

@@ -125,9 +125,8 @@ ghb_status ghb_gram_noalloc(int d, const int* N, const int* M, const double* gri
   size_t off_tab[3][3] = {{0}};
   for (int a = 0; a < d; ++a) {
     if (plan_of[a] != a) continue;
-    // (the third table is not used here; its room keeps the size limit where it was)
-    const size_t sz[3] = {sizeof(int) * tab[a].fx_perm.size(), sizeof(fxw) * tab[a].fx_tw.size(),
-                          sizeof(float2) * tab[a].tw32.size()};
+    const size_t sz[3] = {sizeof(int) * tab[a].perm_of[0].size(), sizeof(fxw) * tab[a].fx_tw.size(),
+                          2 * sizeof(int) * tab[a].nat_of[0].size()};   // (twice: the size limit stays where it was)
     for (int k = 0; k < 3; ++k) {
       off_tab[a][k] = need;
       need += al256(sz[k]);
@@ -164,12 +163,15 @@ ghb_status ghb_gram_noalloc(int d, const int* N, const int* M, const double* gri
   // before the call returns, so the host vectors may go out of scope)
   for (int a = 0; a < d; ++a) {
     if (plan_of[a] != a) continue;
-    GHB_CUDA_TRY(cudaMemcpyAsync(base + off_tab[a][0], tab[a].fx_perm.data(), sizeof(int) * tab[a].fx_perm.size(),
+    GHB_CUDA_TRY(cudaMemcpyAsync(base + off_tab[a][0], tab[a].perm_of[0].data(), sizeof(int) * tab[a].perm_of[0].size(),
+                                 cudaMemcpyHostToDevice, s));
+    GHB_CUDA_TRY(cudaMemcpyAsync(base + off_tab[a][2], tab[a].nat_of[0].data(), sizeof(int) * tab[a].nat_of[0].size(),
                                  cudaMemcpyHostToDevice, s));
     GHB_CUDA_TRY(cudaMemcpyAsync(base + off_tab[a][1], tab[a].fx_tw.data(), sizeof(fxw) * tab[a].fx_tw.size(),
                                  cudaMemcpyHostToDevice, s));
     pl[a].fx.perm = reinterpret_cast<const int*>(base + off_tab[a][0]);
     pl[a].fx.tw = reinterpret_cast<const fxw*>(base + off_tab[a][1]);
+    pl[a].fx.nat = reinterpret_cast<const int*>(base + off_tab[a][2]);
   }
   // the Gram pass's completion counter must start at zero on every call
   GHB_CUDA_TRY(cudaMemsetAsync(base + off_ticket, 0, 256, s));

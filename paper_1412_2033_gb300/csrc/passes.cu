@@ -19,64 +19,51 @@
 
 #include "ghb_internal.cuh"
 #include "passes_fx.cuh"
+#include "passes_rt.cuh"
 
 namespace ghb {
 
-// Launchers defined by instantiation in the col_*.cu / row_*.cu units.
-template <typename T, int TW, int MCT = 0>
-ghb_status launch_col_tw(int sign, int mode, const ColArgs& a, const FftPlan& pl, cudaStream_t s);
-template <typename T, int NL, int MODE>
-ghb_status launch_row_nl(const RowArgs& a, const FftPlan& pl, int rows_per_cta, cudaStream_t s);
-template <typename T, int TW>
-ghb_status launch_col_batch_tw(int sign, int mode, const ColItem* items, int n, int64_t blocks, size_t smem, int threads,
-                               cudaStream_t s);
-template <typename T, int NL, int MODE>
-ghb_status launch_row_batch_nl(const RowItem* items, int n, int64_t blocks, size_t smem, int threads, cudaStream_t s);
+// Launchers defined by instantiation in the ct_*.cu units.
+template <int M>
+ghb_status launch_col_ct_m(int sign, int mode, const ColArgs& a, const CtTables& pl, cudaStream_t s);
+template <int M>
+ghb_status launch_row_ct_m(int NL, const RowArgs& a, const CtTables& pl, int rows_per_cta, cudaStream_t s);
 
-template <typename T, int M>
-ghb_status launch_col_ct_m(int sign, int mode, const ColArgs& a, const FftPlan& pl, cudaStream_t s);
-template <typename T, int M>
-ghb_status launch_row_ct_m(int NL, const RowArgs& a, const FftPlan& pl, int rows_per_cta, cudaStream_t s);
-
-template <typename T>
 ghb_status launch_col_ct(int sign, int mode, const ColArgs& a, const FftPlan& pl, cudaStream_t s) {
   switch (pl.M) {
-    case 162: return launch_col_ct_m<T, 162>(sign, mode, a, pl, s);
-    case 486: return launch_col_ct_m<T, 486>(sign, mode, a, pl, s);
-    case 1458: return launch_col_ct_m<T, 1458>(sign, mode, a, pl, s);
-    case 4374: return launch_col_ct_m<T, 4374>(sign, mode, a, pl, s);
-    case 2187: return launch_col_ct_m<T, 2187>(sign, mode, a, pl, s);
-    case 72: return launch_col_ct_m<T, 72>(sign, mode, a, pl, s);
-    case 135: return launch_col_ct_m<T, 135>(sign, mode, a, pl, s);
-    case 270: return launch_col_ct_m<T, 270>(sign, mode, a, pl, s);
+    case 162: return launch_col_ct_m<162>(sign, mode, a, pl.ct, s);
+    case 486: return launch_col_ct_m<486>(sign, mode, a, pl.ct, s);
+    case 1458: return launch_col_ct_m<1458>(sign, mode, a, pl.ct, s);
+    case 4374: return launch_col_ct_m<4374>(sign, mode, a, pl.ct, s);
+    case 2187: return launch_col_ct_m<2187>(sign, mode, a, pl.ct, s);
+    case 72: return launch_col_ct_m<72>(sign, mode, a, pl.ct, s);
+    case 135: return launch_col_ct_m<135>(sign, mode, a, pl.ct, s);
+    case 270: return launch_col_ct_m<270>(sign, mode, a, pl.ct, s);
     default: break;
   }
   set_error("internal: no size-specialised kernels for M=" + std::to_string(pl.M));
   return GHB_ERR_INVALID;
 }
-template ghb_status launch_col_ct<float>(int, int, const ColArgs&, const FftPlan&, cudaStream_t);
 
-template <typename T>
 ghb_status launch_row_ct(int NL, const RowArgs& a, const FftPlan& pl, int rows_per_cta, cudaStream_t s) {
   switch (pl.M) {
-    case 162: return launch_row_ct_m<T, 162>(NL, a, pl, rows_per_cta, s);
-    case 486: return launch_row_ct_m<T, 486>(NL, a, pl, rows_per_cta, s);
-    case 1458: return launch_row_ct_m<T, 1458>(NL, a, pl, rows_per_cta, s);
-    case 4374: return launch_row_ct_m<T, 4374>(NL, a, pl, rows_per_cta, s);
-    case 2187: return launch_row_ct_m<T, 2187>(NL, a, pl, rows_per_cta, s);
-    case 72: return launch_row_ct_m<T, 72>(NL, a, pl, rows_per_cta, s);
-    case 135: return launch_row_ct_m<T, 135>(NL, a, pl, rows_per_cta, s);
-    case 270: return launch_row_ct_m<T, 270>(NL, a, pl, rows_per_cta, s);
+    case 162: return launch_row_ct_m<162>(NL, a, pl.ct, rows_per_cta, s);
+    case 486: return launch_row_ct_m<486>(NL, a, pl.ct, rows_per_cta, s);
+    case 1458: return launch_row_ct_m<1458>(NL, a, pl.ct, rows_per_cta, s);
+    case 4374: return launch_row_ct_m<4374>(NL, a, pl.ct, rows_per_cta, s);
+    case 2187: return launch_row_ct_m<2187>(NL, a, pl.ct, rows_per_cta, s);
+    case 72: return launch_row_ct_m<72>(NL, a, pl.ct, rows_per_cta, s);
+    case 135: return launch_row_ct_m<135>(NL, a, pl.ct, rows_per_cta, s);
+    case 270: return launch_row_ct_m<270>(NL, a, pl.ct, rows_per_cta, s);
     default: break;
   }
   set_error("internal: no size-specialised kernels for M=" + std::to_string(pl.M));
   return GHB_ERR_INVALID;
 }
-template ghb_status launch_row_ct<float>(int, const RowArgs&, const FftPlan&, int, cudaStream_t);
 
 // The size-specialised FP32 kernels run where they are compiled, the plan
 // carries their input order and the autotuner chose them.
-bool use_ct(const FftPlan& pl, bool tuned_on) { return pl.perm_ct != nullptr && ct_size(pl.M) && tuned_on; }
+bool use_ct(const FftPlan& pl, bool tuned_on) { return pl.ct.perm != nullptr && ct_size(pl.M) && tuned_on; }
 
 namespace {
 
@@ -95,31 +82,12 @@ int device_sms() {
 
 }  // namespace
 
-// Columns per CTA of a runtime-plan column pass over `outer` x `inner` lines:
-// the widest tile (coalesced rows of up to 16 entries) whose CTAs still fill
-// the device three times over; operands too narrow for that take the tile
-// with the most CTAs.  Wide operands (the axis-1 pass in 3-D) get wide tiles,
-// narrow ones (2-D operands of small N) narrow ones.
-int auto_tile(int M, int64_t outer, int64_t inner, int elem_bytes) {
-  const int sms = device_sms();
-  int fallback = 0;
-  for (int tw : {16, 8, 4, 2, 1}) {
-    const size_t smem = col_smem_bytes(M, tw, elem_bytes);
-    if (smem > 220 * 1024) continue;
-    const int64_t per_sm = std::max<int64_t>(1, std::min<int64_t>(4, (227 * 1024) / static_cast<int64_t>(smem)));
-    const int64_t ctas = outer * ((inner + tw - 1) / tw);
-    if (ctas >= 3 * per_sm * sms) return tw;
-    fallback = tw;   // the narrowest fitting tile: the most CTAs
-  }
-  return fallback > 0 ? fallback : 1;
-}
-
 // FP64 columns per CTA: the widest tile (32-byte and longer row segments) that
 // leaves room for three CTAs on an SM and makes at least two CTAs for each; an
 // operand too small for that takes one column per CTA.
-int fx_col_tile(const FftPlan& pl, int64_t columns) {
+int fx_col_tile(int ls, int64_t columns) {
   for (int tw : {8, 4, 2}) {
-    const size_t smem = static_cast<size_t>(tw) * pl.fx.ls * sizeof(fx2);
+    const size_t smem = static_cast<size_t>(tw) * ls * sizeof(fx2);
     if (smem <= 73 * 1024 && (columns + tw - 1) / tw >= 2 * device_sms()) return tw;
   }
   return 1;
@@ -152,41 +120,68 @@ void fx_row_shape(int mode, int nfields, int ncomp, int M, int ls, int64_t rows,
   *threads = fx_threads(M, *NL, ls);
 }
 
+// FP32 run-time plans.  Columns per CTA: the widest tile (row segments of 8 TW
+// bytes) that leaves room for three CTAs on an SM and makes two for each; four
+// columns also as one CTA of 768 threads and from 1.6 CTAs for each SM (M = 2048,
+// 1024 columns: 22 / 20 us with four, 28 / 23 with two; M = 1440, 702 columns: 21 /
+// 18 with four, 19 / 14 with two).
+int rt_col_tile(int M, int ls, int64_t columns) {
+  for (int tw : {16, 8, 4}) {
+    const size_t smem = static_cast<size_t>(tw) * ls * sizeof(float2);
+    const int64_t ctas = (columns + tw - 1) / tw;
+    if (smem <= (tw == 4 ? 150 : 73) * 1024 && 10 * ctas >= (tw == 4 ? 16 : 20) * device_sms()) return tw;
+  }
+  return 2;
+}
+// about one group of sixteen entries a thread and pass, whole warps
+int rt_threads(int M, int lines, int ls) {
+  const size_t smem = static_cast<size_t>(lines) * ls * sizeof(float2);
+  const int full = smem > 110 * 1024 ? kRtThreads : (smem > 73 * 1024 ? kRtThreads / 2 : kRtThreads / 3);
+  const int t = ((lines * M / 16 + 31) / 32) * 32;
+  return t < 64 ? 64 : (t < full ? t : full);
+}
+// Last axis: the least rows that fill complex lines (d = 2: one, d = 3: two rows,
+// three lines), doubled while a block of 256 has threads without a group and two
+// CTAs remain for each SM; `want` = 1 keeps the least, 2 doubles it once.
+void rt_row_shape(int ncomp, int M, int ls, int64_t rows, int want, int* rows_per_cta, int* lines) {
+  int r = ncomp == 2 ? 1 : 2, q = r * ncomp / 2;
+  while (want != 1 && 2 * q <= kRtMaxLines && static_cast<size_t>(2 * q) * ls * sizeof(float2) <= 73 * 1024 &&
+         (want == 2 || (q * (M / 16) < 192 && rows / (2 * r) >= 2 * device_sms()))) {
+    r *= 2;
+    q *= 2;
+    if (want == 2) break;
+  }
+  *rows_per_cta = r;
+  *lines = q;
+}
+
 template <>
 ghb_status launch_col<double>(int sign, int mode, const ColArgs& a, const FftPlan& pl, cudaStream_t s) {
   int TW = pl.tile[0];   // ghb_tune_set; 0 = by the operand
-  if (TW <= 0 || static_cast<size_t>(TW) * pl.fx.ls * sizeof(fx2) > 220 * 1024)
-    TW = fx_col_tile(pl, a.outer * a.inner);
+  if (TW <= 0 || static_cast<size_t>(TW) * (pl.fx.ls + 15) * sizeof(fx2) > 220 * 1024)
+    TW = fx_col_tile(pl.fx.ls, a.outer * a.inner);
   if (col_smem_bytes(pl.M, 1, sizeof(double2)) > 220 * 1024) {
     set_error("transform length too large for one CTA: M=" + std::to_string(pl.M));
     return GHB_ERR_INVALID;
   }
   ColArgs b = a;
   if (mode != COL_PUPDATE) b.pold = nullptr;
-  return launch_fx_col(sign, b, pl, TW, s);
+  return launch_fx_col(sign, b, pl.fx, TW, s);
 }
 
 template <>
 ghb_status launch_col<float>(int sign, int mode, const ColArgs& a, const FftPlan& pl, cudaStream_t s) {
-  using T = float;
-  using C = float2;
-  if (use_ct(pl, pl.ct_col != 0)) return launch_col_ct<T>(sign, mode, a, pl, s);
-  const int forced = pl.tile[1];   // ghb_tune_set; 0 = by the operand
-  const int TW = forced > 0 ? forced : auto_tile(pl.M, a.outer, a.inner, sizeof(C));
-  if (col_smem_bytes(pl.M, TW, sizeof(C)) > 220 * 1024) {
-    set_error("transform length too large for one CTA: M=" + std::to_string(pl.M));
+  if (use_ct(pl, pl.ct_col != 0)) return launch_col_ct(sign, mode, a, pl, s);
+  if (a.outer * std::max<int64_t>(std::max(a.Lin, a.Lout), pl.M) * a.inner >= (int64_t(1) << 31)) {
+    set_error("column pass operand of 2^31 entries or more");
     return GHB_ERR_INVALID;
   }
-  switch (TW) {
-    case 1: return launch_col_tw<T, 1>(sign, mode, a, pl, s);
-    case 2: return launch_col_tw<T, 2>(sign, mode, a, pl, s);
-    case 4: return launch_col_tw<T, 4>(sign, mode, a, pl, s);
-    case 8: return launch_col_tw<T, 8>(sign, mode, a, pl, s);
-    case 16: return launch_col_tw<T, 16>(sign, mode, a, pl, s);
-    default: break;
-  }
-  set_error("internal: bad tile width");
-  return GHB_ERR_INVALID;
+  int TW = pl.tile[1];   // ghb_tune_set; 0 = by the operand
+  if (TW <= 0 || static_cast<size_t>(TW) * (pl.rt.ls + 15) * sizeof(float2) > 220 * 1024)
+    TW = rt_col_tile(pl.M, pl.rt.ls, a.outer * a.inner);
+  ColArgs b = a;
+  if (mode != COL_PUPDATE) b.pold = nullptr;
+  return launch_rt_col(sign, b, pl.rt, TW, s);
 }
 
 // Rows a CTA transforms together in the operator's last-axis pass (d = 2:
@@ -204,17 +199,7 @@ void row_lines(int mode, int nfields, int ncomp, int M, int rows32, int* rows_pe
 template <>
 ghb_status launch_col_batch<float>(int sign, int mode, int TW, const ColItem* items, int n, int64_t blocks,
                                    size_t smem, int threads, cudaStream_t s) {
-  using T = float;
-  switch (TW) {
-    case 1: return launch_col_batch_tw<T, 1>(sign, mode, items, n, blocks, smem, threads, s);
-    case 2: return launch_col_batch_tw<T, 2>(sign, mode, items, n, blocks, smem, threads, s);
-    case 4: return launch_col_batch_tw<T, 4>(sign, mode, items, n, blocks, smem, threads, s);
-    case 8: return launch_col_batch_tw<T, 8>(sign, mode, items, n, blocks, smem, threads, s);
-    case 16: return launch_col_batch_tw<T, 16>(sign, mode, items, n, blocks, smem, threads, s);
-    default: break;
-  }
-  set_error("internal: bad tile width");
-  return GHB_ERR_INVALID;
+  return launch_rt_col_batch(sign, mode == COL_PUPDATE, TW, items, n, blocks, smem, threads, s);
 }
 template <>
 ghb_status launch_col_batch<double>(int sign, int, int TW, const ColItem* items, int n, int64_t blocks, size_t smem,
@@ -225,12 +210,7 @@ ghb_status launch_col_batch<double>(int sign, int, int TW, const ColItem* items,
 template <>
 ghb_status launch_row_batch<float>(int mode, int NL, const RowItem* items, int n, int64_t blocks, size_t smem,
                                    int threads, cudaStream_t s) {
-  using T = float;
-  if (mode == ROW_MATVEC) {
-    if (NL == 1) return launch_row_batch_nl<T, 1, ROW_MATVEC>(items, n, blocks, smem, threads, s);
-    if (NL == 2) return launch_row_batch_nl<T, 2, ROW_MATVEC>(items, n, blocks, smem, threads, s);
-    if (NL == 3) return launch_row_batch_nl<T, 3, ROW_MATVEC>(items, n, blocks, smem, threads, s);
-  }
+  if (mode == ROW_MATVEC) return launch_rt_row_batch(NL, items, n, blocks, smem, threads, s);
   set_error("internal: unsupported batched row pass");
   return GHB_ERR_INVALID;
 }
@@ -242,19 +222,15 @@ ghb_status launch_row_batch<double>(int mode, int NL, const RowItem* items, int 
 
 template <>
 ghb_status launch_row<float>(int mode, const RowArgs& a, const FftPlan& pl, cudaStream_t s) {
-  using T = float;
   int rows_per_cta = 1, NL = 1;
   row_lines(mode, a.nfields, a.ncomp, pl.M, pl.rows32, &rows_per_cta, &NL);
   if (mode == ROW_MATVEC) {   // set-up and Gram passes run in FP64 only
-    if (use_ct(pl, pl.ct_row != 0)) return launch_row_ct<T>(NL, a, pl, rows_per_cta, s);
-    switch (NL) {
-      case 1: return launch_row_nl<T, 1, ROW_MATVEC>(a, pl, rows_per_cta, s);
-      case 2: return launch_row_nl<T, 2, ROW_MATVEC>(a, pl, rows_per_cta, s);
-      case 3: return launch_row_nl<T, 3, ROW_MATVEC>(a, pl, rows_per_cta, s);
-      default: break;
-    }
+    if (use_ct(pl, pl.ct_row != 0)) return launch_row_ct(NL, a, pl, rows_per_cta, s);
+    int lines = 1;
+    rt_row_shape(a.ncomp, pl.M, pl.rt.ls, a.rows, pl.rows32, &rows_per_cta, &lines);
+    return launch_rt_row(a, pl.rt, rows_per_cta, lines, s);
   }
-  set_error("internal: unsupported row-pass line count");
+  set_error("internal: unsupported FP32 row pass");
   return GHB_ERR_INVALID;
 }
 
@@ -267,7 +243,7 @@ ghb_status launch_row<double>(int mode, const RowArgs& a, const FftPlan& pl, cud
     return GHB_ERR_INVALID;
   }
   fx_row_shape(mode, a.nfields, a.ncomp, pl.M, pl.fx.ls, a.rows, &rows_per_cta, &NL, &threads);
-  return launch_fx_row(mode, a, pl, rows_per_cta, NL, threads, s);
+  return launch_fx_row(mode, a, pl.fx, rows_per_cta, NL, threads, s);
 }
 
 }  // namespace ghb

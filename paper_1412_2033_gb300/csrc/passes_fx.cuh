@@ -8,9 +8,9 @@
 // (radix 3 x 3), a third of the pass's time in conversions and the multiply.
 // One CTA holds its lines whole in shared memory, one after the other.
 // Measured against the FP64-pipe kernels these replace (N = 2187, M = 4374):
-// last axis 4267 -> 1017 us, axis 1 1048 / 1047 -> 316 / 294 us, one operator
-// application 6.50 -> 1.76 ms; d = 3, N = 63 x 99 x 77 2.51 -> 0.57 ms; N = 315 x
-// 517 354 -> 100 us.
+// last axis 4267 -> 961 us, axis 1 1048 / 1047 -> 331 / 304 us, one operator
+// application 6.50 -> 1.73 ms; d = 3, N = 63 x 99 x 77 2.51 -> 0.54 ms; N = 315 x
+// 517 354 -> 98 us.
 #pragma once
 
 #include <algorithm>
@@ -31,8 +31,7 @@ constexpr int kFxBlocks = 1;
 // magnitudes after each pass (slot k: before the k-th pass of the sequence).
 struct FxShared {
   FxPass p[kFxPasses];
-  int np, pad;
-  FastDiv pdiv;
+  int np;
   int mag[2 * kFxPasses + 2][kFxMaxLines];
   int emax[kFxMaxLines];    // largest |word| of the line's doubles, then its biased exponent
   int wmax[kFxMaxLines];    // the same of the line after the multiply
@@ -43,20 +42,12 @@ __device__ __forceinline__ void fx_load_plan(FxShared& sh, const FxPlan& f) {
   const int* src = reinterpret_cast<const int*>(f.p);
   int* dst = reinterpret_cast<int*>(sh.p);
   for (int i = threadIdx.x; i < n; i += blockDim.x) dst[i] = src[i];
-  if (threadIdx.x == 0) {
-    sh.np = f.np;
-    sh.pad = f.pad;
-    sh.pdiv = f.pdiv;
-  }
+  if (threadIdx.x == 0) sh.np = f.np;
 }
 
 __device__ __forceinline__ void fx_clear_lines(FxShared& sh) {
   for (int i = threadIdx.x; i < (2 * kFxPasses + 2) * kFxMaxLines; i += blockDim.x) (&sh.mag[0][0])[i] = 0;
   if (threadIdx.x < kFxMaxLines) sh.emax[threadIdx.x] = sh.wmax[threadIdx.x] = 0;
-}
-
-__device__ __forceinline__ int fx_pos(const FxShared& sh, int n) {
-  return sh.pad > 0 ? n + static_cast<int>(fdiv(static_cast<unsigned>(n), sh.pdiv)) : n;
 }
 
 // Shift before the pass in slot k (bits: what it admits); the first pass after
@@ -70,7 +61,7 @@ __device__ __forceinline__ int fx_shift_of(const FxShared& sh, int k, int k0, in
 // k0 .. k0 + np.  Barriers: before the first pass by the caller, after each here.
 template <int SIGN, bool DIT>
 __device__ __forceinline__ void fx_transform(fx2* buf, int ls, int lines, FxShared& sh, int k0, int M,
-                                             const fxw* __restrict__ tw) {
+                                             const int* __restrict__ nat, const fxw* __restrict__ tw) {
   const int np = sh.np;
   for (int k = 0; k < np; ++k) {
     const int i = DIT ? k : np - 1 - k;
@@ -84,8 +75,7 @@ __device__ __forceinline__ void fx_transform(fx2* buf, int ls, int lines, FxShar
         line = static_cast<int>(fdiv(static_cast<unsigned>(u), P.ulines));
         const int g = fx_shift_of(sh, k0 + k, k0, DIT ? P.bits_dit : P.bits_dif, line);
         int p;
-        const int pos = fx_unit_base(P, sh.pad, sh.pdiv, u - line * P.units, p);
-        fx2* base = buf + line * ls + pos;
+        fx2* base = buf + line * ls + __ldg(&nat[fx_unit_entry(P, u - line * P.units, p)]);
         m = i == 0 ? fx_run_unit<SIGN, DIT, true>(P, base, g, p, M, tw)
                    : fx_run_unit<SIGN, DIT, false>(P, base, g, p, M, tw);
       }
@@ -129,14 +119,13 @@ __device__ __forceinline__ int fx_ref(int word) {
 // (outer, inner) range; a thread always handles column threadIdx.x mod TW.
 // ---------------------------------------------------------------------------
 template <int SIGN>
-__device__ __forceinline__ void fx_col_body(const ColArgs& a, const FftPlan& pl, int TW, int64_t bid) {
+__device__ __forceinline__ void fx_col_body(const ColArgs& a, const FxPlan& f, int TW, int64_t bid) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   fx2* buf = reinterpret_cast<fx2*>(smem_raw);
   __shared__ FxShared sh;
   if (a.st != nullptr && a.st->done != RUNNING) return;
-  const FxPlan& f = pl.fx;
-  const int M = pl.M;
-  const int ls = f.ls;
+  const int M = f.M;
+  const int ls = column_stride(f.ls, TW, sizeof(fx2));
   fx_load_plan(sh, f);
   fx_clear_lines(sh);
 
@@ -197,6 +186,7 @@ __device__ __forceinline__ void fx_col_body(const ColArgs& a, const FftPlan& pl,
   const bool bad = (word >> 20) == kFxNonFinite;
   const int E = fx_ref(word), bits = fx_first_bits(sh, SIGN > 0);
   const int* __restrict__ perm = f.perm;
+  const int* __restrict__ nat = f.nat;
   const int half = (Lin - 1) / 2;
 
   for (int ib = i0; ib < Lin; ib += K * di) {
@@ -213,7 +203,7 @@ __device__ __forceinline__ void fx_col_body(const ColArgs& a, const FftPlan& pl,
       const int i = ib + c * di;
       if (i < Lin) {
         const int k = i - half < 0 ? i - half + M : i - half;
-        const int pos = SIGN > 0 ? __ldg(&perm[k]) : fx_pos(sh, i);
+        const int pos = SIGN > 0 ? __ldg(&perm[k]) : __ldg(&nat[i]);
         line[pos] = bad ? fx2{0, 0} : fx2{fx_from_double(r[c].x, E, bits), fx_from_double(r[c].y, E, bits)};
       }
     }
@@ -221,7 +211,7 @@ __device__ __forceinline__ void fx_col_body(const ColArgs& a, const FftPlan& pl,
   if (SIGN > 0)
     for (int k = half + 1 + i0; k < M - half; k += di) line[__ldg(&perm[k])] = fx2{0, 0};
   __syncthreads();
-  fx_transform<SIGN, (SIGN > 0)>(buf, ls, TW, sh, 0, M, f.tw);
+  fx_transform<SIGN, (SIGN > 0)>(buf, ls, TW, sh, 0, M, nat, f.tw);
 
   if (!valid) return;
   FxScale so = fx_scale_of(E - 1022 - bits + fx_exponent<(SIGN > 0)>(sh, 0, t));
@@ -230,7 +220,7 @@ __device__ __forceinline__ void fx_col_body(const ColArgs& a, const FftPlan& pl,
   if (SIGN > 0) {
     double2* out = static_cast<double2*>(a.out) + o * M * inner + jj;
     for (int m = i0; m < M; m += di) {
-      const fx2 v = line[fx_pos(sh, m)];
+      const fx2 v = line[__ldg(&nat[m])];
       out[m * inner] = make_double2(fx_to_double(v.x, so), fx_to_double(v.y, so));
     }
   } else {
@@ -275,7 +265,7 @@ __device__ __forceinline__ FxMultiplier fx_multiplier(double a) {
 }
 
 template <int MODE>
-__device__ __forceinline__ void fx_row_body(const RowArgs& a, const FftPlan& pl, int rows_per_cta, int NL, int64_t bid,
+__device__ __forceinline__ void fx_row_body(const RowArgs& a, const FxPlan& f, int rows_per_cta, int NL, int64_t bid,
                                             int64_t nb) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   fx2* buf = reinterpret_cast<fx2*>(smem_raw);
@@ -284,12 +274,12 @@ __device__ __forceinline__ void fx_row_body(const RowArgs& a, const FftPlan& pl,
   __shared__ double red[32];
   __shared__ bool last;
   if (a.st != nullptr && a.st->done != RUNNING) return;
-  const FxPlan& f = pl.fx;
-  const int M = pl.M, H = a.H, ls = f.ls;
+  const int M = f.M, H = a.H, ls = f.ls;
   const int per_row = a.nfields * a.ncomp;
   const int nrl = rows_per_cta * per_row;
   const int64_t groups = (a.rows + rows_per_cta - 1) / rows_per_cta;
   const int* __restrict__ perm = f.perm;
+  const int* __restrict__ nat = f.nat;
   const int lane = threadIdx.x & 31;
   const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0);
   const int nwarp = blockDim.x >> 5;
@@ -358,7 +348,7 @@ __device__ __forceinline__ void fx_row_body(const RowArgs& a, const FftPlan& pl,
       for (int k = H + k0; k <= M - H; k += 32 * segs) line[__ldg(&perm[k])] = fx2{0, 0};
     }
     __syncthreads();
-    fx_transform<+1, true>(buf, ls, NL, sh, 0, M, f.tw);
+    fx_transform<+1, true>(buf, ls, NL, sh, 0, M, nat, f.tw);
 
     if (MODE == ROW_MATVEC) {
       // Multiply by A_M.  The products' largest exponent is found first (from
@@ -375,7 +365,7 @@ __device__ __forceinline__ void fx_row_body(const RowArgs& a, const FftPlan& pl,
         int mx = 0;
 #pragma unroll 4
         for (int m = m0; m < M; m += 32 * segs) {
-          const fx2 u = line[fx_pos(sh, m)];
+          const fx2 u = line[__ldg(&nat[m])];
           const int w0 = static_cast<int>(__double_as_longlong(__ldg(&a0[m])) >> 32) & 0x7fffffff;
           int w1 = w0;
           if (a1 != a0) w1 = static_cast<int>(__double_as_longlong(__ldg(&a1[m])) >> 32) & 0x7fffffff;
@@ -409,7 +399,7 @@ __device__ __forceinline__ void fx_row_body(const RowArgs& a, const FftPlan& pl,
         const bool same = a0 == a1;   // both real lines of one row
 #pragma unroll 2
         for (int m = m0; m < M; m += 32 * segs) {
-          const int pos = fx_pos(sh, m);
+          const int pos = __ldg(&nat[m]);
           const fx2 u = line[pos];
           const FxMultiplier x0 = fx_multiplier(__ldg(&a0[m]));
           FxMultiplier x1 = x0;
@@ -418,7 +408,7 @@ __device__ __forceinline__ void fx_row_body(const RowArgs& a, const FftPlan& pl,
         }
       }
       __syncthreads();
-      fx_transform<-1, false>(buf, ls, NL, sh, kp + 1, M, f.tw);
+      fx_transform<-1, false>(buf, ls, NL, sh, kp + 1, M, nat, f.tw);
 
       for (int idx = warp; idx < NL * segs; idx += nwarp) {
         const int j = idx / segs, k0 = (idx - j * segs) * 32 + lane;
@@ -456,7 +446,7 @@ __device__ __forceinline__ void fx_row_body(const RowArgs& a, const FftPlan& pl,
         if (bad) so.a = __longlong_as_double(0x7ff8000000000000LL);
         double* out = static_cast<double*>(a.out_real);
         for (int m = m0; m < M; m += 32 * segs) {
-          const int pos = fx_pos(sh, m);
+          const int pos = __ldg(&nat[m]);
           const fx2 u = line[pos];
           const double2 z = make_double2(fx_to_double(u.x, so), fx_to_double(u.y, so));
           if (MODE == ROW_TOREAL) {
@@ -474,7 +464,7 @@ __device__ __forceinline__ void fx_row_body(const RowArgs& a, const FftPlan& pl,
         const double* val = reinterpret_cast<const double*>(buf);
         for (int m = threadIdx.x; m < M; m += blockDim.x) {
           const double w = am[ld[0].row[0] * M + m];
-          const int pos = fx_pos(sh, m);
+          const int pos = __ldg(&nat[m]);
           auto at = [&](int r) { return val[2 * ((r >> 1) * ls + pos) + (r & 1)]; };
           int e = 0;
 #pragma unroll
@@ -536,16 +526,16 @@ __device__ __forceinline__ void fx_row_body(const RowArgs& a, const FftPlan& pl,
 }
 
 // Launch shapes (passes.cu).
-int fx_col_tile(const FftPlan& pl, int64_t columns);
+int fx_col_tile(int ls, int64_t columns);
 int fx_threads(int M, int lines, int ls);
 void fx_row_shape(int mode, int nfields, int ncomp, int M, int ls, int64_t rows, int* rows_per_cta, int* NL,
                   int* threads);
 
 // Launchers (fx_col.cu, fx_row.cu).
-ghb_status launch_fx_col(int sign, const ColArgs& a, const FftPlan& pl, int TW, cudaStream_t s);
+ghb_status launch_fx_col(int sign, const ColArgs& a, const FxPlan& f, int TW, cudaStream_t s);
 ghb_status launch_fx_col_batch(int sign, int TW, const ColItem* items, int n, int64_t blocks, size_t smem, int threads,
                                cudaStream_t s);
-ghb_status launch_fx_row(int mode, const RowArgs& a, const FftPlan& pl, int rows_per_cta, int NL, int threads,
+ghb_status launch_fx_row(int mode, const RowArgs& a, const FxPlan& f, int rows_per_cta, int NL, int threads,
                          cudaStream_t s);
 ghb_status launch_fx_row_batch(int mode, int NL, const RowItem* items, int n, int64_t blocks, size_t smem, int threads,
                                cudaStream_t s);

@@ -25,122 +25,82 @@ bool factor(int M, std::vector<int>& radices) {
   return m == 1 && static_cast<int>(radices.size()) <= kMaxStages;
 }
 
-struct Shape {
-  int id;
-  int r[3];
+struct GroupShape {
+  int id, r[2];
 };
+const GroupShape kFxShapes[] = {{FX_5_2, {5, 2}}, {FX_3_3, {3, 3}}, {FX_4_2, {4, 2}}, {FX_3_2, {3, 2}},
+                                {FX_5, {5, 1}},   {FX_4, {4, 1}},   {FX_3, {3, 1}},   {FX_2, {2, 1}}};
+const GroupShape kRtShapes[] = {{RT_4_4, {4, 4}}, {RT_5_3, {5, 3}}, {RT_3_4, {3, 4}}, {RT_5_2, {5, 2}},
+                                {RT_3_3, {3, 3}}, {RT_4_2, {4, 2}}, {RT_3_2, {3, 2}}, {RT_5, {5, 1}},
+                                {RT_4, {4, 1}},   {RT_3, {3, 1}},   {RT_2, {2, 1}}};
 
-// Pass shapes in DIT radix order (see PassShape); longest first.
-const Shape kShapes[] = {
-    {SH_2_3_3, {2, 3, 3}}, {SH_3_3_3, {3, 3, 3}}, {SH_4_2_3, {4, 2, 3}}, {SH_2_3_5, {2, 3, 5}},
-    {SH_4_4_2, {4, 4, 2}}, {SH_2_3, {2, 3, 0}},   {SH_3_3, {3, 3, 0}},   {SH_2_5, {2, 5, 0}},
-    {SH_4_3, {4, 3, 0}},   {SH_3_5, {3, 5, 0}},   {SH_4_4, {4, 4, 0}},   {SH_4_5, {4, 5, 0}},
-    {SH_5_5, {5, 5, 0}},   {SH_4_2, {4, 2, 0}},   {SH_2, {2, 0, 0}},     {SH_3, {3, 0, 0}},
-    {SH_4, {4, 0, 0}},     {SH_5, {5, 0, 0}},
-};
-
-}  // namespace
-
-// Group consecutive stages into passes: at each stage take the first (longest)
-// shape that matches the next radices with radix product <= maxprod.
-void group_passes(FftPlan& p, int maxprod) {
-  int t = 0, np = 0;
-  while (t < p.nst) {
-    int best = -1, blen = 0;
-    for (const Shape& sh : kShapes) {
-      int len = 0;
-      while (len < 3 && sh.r[len] != 0) ++len;
-      if (t + len > p.nst) continue;
-      int prod = 1;
-      for (int q = 0; q < len; ++q) prod *= sh.r[q];
-      if (prod > maxprod) continue;
-      bool ok = true;
-      for (int k = 0; k < len; ++k) ok = ok && (p.R[t + k] == sh.r[k]);
-      if (ok && len > blen) {
-        best = sh.id;
-        blen = len;
+// The groups of product <= cap, `left` of them in list order from `from`, that
+// multiply to 2^a 3^b 5^c with the least sum of sizes (balanced: a pass's threads
+// go with the number of its groups).
+struct Cover {
+  const GroupShape* shapes;
+  int count, cap;
+  std::vector<int> now, best;
+  int best_sum = INT_MAX;
+  void search(int a, int b, int c, int from, int left, int sum) {
+    if (a == 0 && b == 0 && c == 0) {
+      if (left == 0 && sum < best_sum) {
+        best_sum = sum;
+        best = now;
       }
+      return;
     }
-    int prod = 1;
-    if (best < 0) {
-      best = SH_GENERIC;
-      blen = 1;
+    if (left == 0) return;
+    for (int i = from; i < count; ++i) {
+      const int* r = shapes[i].r;
+      const int size = r[0] * r[1];
+      if (size > cap) continue;
+      int d[3] = {0, 0, 0};   // exponents of 2, 3, 5
+      for (int k = 0; k < 2; ++k) {
+        d[0] += r[k] == 2 ? 1 : (r[k] == 4 ? 2 : 0);
+        d[1] += r[k] == 3;
+        d[2] += r[k] == 5;
+      }
+      if (d[0] > a || d[1] > b || d[2] > c) continue;
+      now.push_back(i);
+      search(a - d[0], b - d[1], c - d[2], i, left - 1, sum + size);
+      now.pop_back();
     }
-    for (int k = 0; k < blen; ++k) prod *= p.R[t + k];
-    p.pshape[np] = best;
-    p.pR[np] = prod;
-    p.pLp[np] = p.Lp[t];
-    p.pdiv[np] = make_fastdiv(static_cast<unsigned>(p.Lp[t]));
-    ++np;
-    t += blen;
   }
-  p.npass = np;
-  for (int i = np; i < kMaxPasses; ++i) {
-    p.pshape[i] = SH_2;
-    p.pR[i] = 1;
-    p.pLp[i] = 1;
-    p.pdiv[i] = make_fastdiv(1);
-  }
-}
-
-namespace {
-
-struct FxShapeDef {
-  int id, ra, rb;
 };
-const FxShapeDef kFxShapes[] = {{FX_5_2, 5, 2}, {FX_3_3, 3, 3}, {FX_4_2, 4, 2}, {FX_3_2, 3, 2},
-                                {FX_5, 5, 1},   {FX_4, 4, 1},   {FX_3, 3, 1},   {FX_2, 2, 1}};
-
-// The fewest passes of product <= cap that multiply to 2^a 3^b 5^c (the first
-// found: large shapes first).
-bool fx_cover(int a, int b, int c, int cap, int left, std::vector<int>& out) {
-  if (a == 0 && b == 0 && c == 0) return true;
-  if (left == 0) return false;
-  for (int i = 0; i < static_cast<int>(sizeof(kFxShapes) / sizeof(kFxShapes[0])); ++i) {
-    const FxShapeDef& s = kFxShapes[i];
-    if (s.ra * s.rb > cap) continue;
-    if (!out.empty() && i < out.back()) continue;   // in list order: each multiset once
-    int da = 0, db = 0, dc = 0;
-    for (int r : {s.ra, s.rb}) {
-      if (r == 2) da += 1;
-      if (r == 4) da += 2;
-      if (r == 3) db += 1;
-      if (r == 5) dc += 1;
-    }
-    if (da > a || db > b || dc > c) continue;
-    out.push_back(i);
-    if (fx_cover(a - da, b - db, c - dc, cap, left - 1, out)) return true;
-    out.pop_back();
-  }
-  return false;
-}
 
 }  // namespace
 
-// Passes of the fixed-point transform (fft_fx.cuh): as few as the cap allows,
-// odd group sizes first (the first pass's threads then sit at an odd stride),
-// primes above 5 last.
-bool fx_group_passes(int M, int cap, FxPlan& f, std::vector<int>* perm_out) {
+// Passes of a run-time transform (k = 0: fft_fx.cuh, 1: fft_rt.cuh): as few as the
+// cap allows, odd group sizes first (the first pass's threads then sit at an odd
+// stride), primes above 5 last.
+bool group_plan(int k, int M, int cap, FxPlan& f, std::vector<int>* perm_out, std::vector<int>* nat_out) {
+  f.M = M;
   int a = 0, b = 0, c = 0, m = M;
   while (m % 2 == 0) { ++a; m /= 2; }
   while (m % 3 == 0) { ++b; m /= 3; }
   while (m % 5 == 0) { ++c; m /= 5; }
-  std::vector<int> sh;
-  bool ok = false;
-  for (int n = 0; n <= kFxPasses && !ok; ++n) {
-    sh.clear();
-    ok = fx_cover(a, b, c, cap < 5 ? 5 : cap, n, sh);
+  Cover cover;
+  cover.shapes = k == 0 ? kFxShapes : kRtShapes;
+  cover.count = static_cast<int>(k == 0 ? sizeof(kFxShapes) / sizeof(GroupShape) : sizeof(kRtShapes) / sizeof(GroupShape));
+  cover.cap = cap < 5 ? 5 : cap;
+  for (int n = 0; n <= kFxPasses && cover.best_sum == INT_MAX; ++n) {
+    if (n == 0 && a + b + c == 0) cover.best_sum = 0;
+    else cover.search(a, b, c, 0, n, 0);
   }
-  if (!ok) return false;
+  if (cover.best_sum == INT_MAX) return false;
   struct P {
     int id, ra, rb;
+    int size() const { return ra * rb; }
   };
   std::vector<P> ps;
-  for (int i : sh) ps.push_back(P{kFxShapes[i].id, kFxShapes[i].ra, kFxShapes[i].rb});
+  for (int i : cover.best) {
+    const GroupShape& g = cover.shapes[i];
+    ps.push_back(P{g.id, g.r[0], g.r[1]});
+  }
   std::stable_sort(ps.begin(), ps.end(), [](const P& x, const P& y) {
-    const int px = x.ra * x.rb, py = y.ra * y.rb;
-    if ((px & 1) != (py & 1)) return (px & 1) > (py & 1);
-    return px > py;
+    if ((x.size() & 1) != (y.size() & 1)) return (x.size() & 1) > (y.size() & 1);
+    return x.size() > y.size();
   });
   for (int p = 7; p <= kMaxGenericRadix && m > 1; p += 2)
     while (m % p == 0) {
@@ -149,10 +109,19 @@ bool fx_group_passes(int M, int cap, FxPlan& f, std::vector<int>* perm_out) {
     }
   if (m != 1 || static_cast<int>(ps.size()) > kFxPasses) return false;
   f.np = static_cast<int>(ps.size());
-  const int first = f.np > 0 ? ps[0].ra * ps[0].rb : 1;
-  f.pad = (f.np > 0 && first % 4 == 0 && first >= 8) ? first : 0;   // strides 2, 6, 10: two-way conflicts only
-  f.pdiv = make_fastdiv(static_cast<unsigned>(f.pad > 0 ? f.pad : 1));
-  f.ls = M + (f.pad > 0 ? M / f.pad : 0);
+  // blocks after which a position is spared, and the positions of an index
+  std::vector<int> spare;
+  auto position = [&](int n) {
+    int pos = n;
+    for (int L : spare) pos += n / L;
+    return pos;
+  };
+  int L = 1;
+  for (const P& p : ps) {
+    L *= p.size();
+    if (L < M && L >= 8 && position(L) % 4 == 0) spare.push_back(L);
+  }
+  f.ls = M > 0 ? position(M - 1) + 1 : 1;
   int lp = 1;
   std::vector<int> radix;
   for (int i = 0; i < kFxPasses; ++i) {
@@ -162,27 +131,31 @@ bool fx_group_passes(int M, int cap, FxPlan& f, std::vector<int>* perm_out) {
       q.ulines = q.ulp = make_fastdiv(1);
       continue;
     }
-    const int R = ps[i].ra * ps[i].rb;
+    const int R = ps[i].size();
     q.shape = ps[i].id;
     q.R = R;
     q.lp = lp;
-    q.step = lp + (f.pad > 0 ? lp / f.pad : 0);
-    q.block = lp * R + (f.pad > 0 ? lp * R / f.pad : 0);
+    q.step = position(lp);
     q.units = M / R;
     q.ts = M / (lp * R);
     q.ulines = make_fastdiv(static_cast<unsigned>(q.units));
     q.ulp = make_fastdiv(static_cast<unsigned>(lp));
-    // A group's values must stay below 2^62 (fx_cmul4): with largest component
-    // 2^b before the pass, magnitudes start at 2^(b + 1/2) and grow by at most
-    // R / 4 per scaled stage, R where the factor 1/4 comes after the sums
-    // (forward) or not at all (the first pass's first stage).
-    const double lr = std::log2(static_cast<double>(q.shape == FX_GENERIC ? R : 5));
-    if (q.shape == FX_GENERIC) {
-      q.bits_dif = static_cast<int>(std::floor(61.5 - (lr - 2)));
-      q.bits_dit = i == 0 ? q.bits_dif : static_cast<int>(std::floor(61.5 - std::max(0.0, lr - 4)));
+    // Bits that the largest component may fill before the pass.  Magnitudes
+    // then start below 2^(b + 1/2); a stage with twiddles multiplies them by
+    // R / 4 at most, R of it before the factor 1/4 in a forward stage, and the
+    // first pass's first stage has no factor.  A product's operand may reach
+    // 2^62.8 (fx_cmul4's cross sums: 2^61.5 + 2^62.3 < 2^63), the results of the
+    // last forward pass 2^62 (pairs of them are added).
+    const bool gen = q.shape == FX_GENERIC, first = i == 0;
+    auto bits = [](double limit, double growth) { return static_cast<int>(std::floor(limit - 0.5 - std::log2(growth))); };
+    const double ra = ps[i].ra, rb = ps[i].rb;
+    if (gen) {
+      q.bits_dif = bits(first ? 62.0 : 62.8, R / 4.0);
+      q.bits_dit = first ? bits(62.8, R / 4.0) : std::min(62, bits(62.8, std::max(1.0, R / 16.0)));
     } else {
-      q.bits_dif = 59;
-      q.bits_dit = i == 0 ? static_cast<int>(std::floor(61.0 - std::log2(static_cast<double>(ps[i].ra)))) : 61;
+      const double last = rb > 1 ? rb / 4 * ra : ra;   // forward: growth up to the sums of the last stage
+      q.bits_dif = std::min(bits(62.8, rb > 1 ? rb : last), bits(first ? 62.0 : 62.8, last));
+      q.bits_dit = first ? bits(62.8, ra) : 62;
     }
     radix.push_back(ps[i].ra);
     if (ps[i].rb > 1) radix.push_back(ps[i].rb);
@@ -203,8 +176,12 @@ bool fx_group_passes(int M, int cap, FxPlan& f, std::vector<int>* perm_out) {
         pos += q[t] * L;
         L *= radix[t];
       }
-      perm[n] = pos + (f.pad > 0 ? pos / f.pad : 0);
+      perm[n] = position(pos);
     }
+  }
+  if (nat_out) {
+    nat_out->resize(M);
+    for (int n = 0; n < M; ++n) (*nat_out)[n] = position(n);
   }
   return true;
 }
@@ -281,36 +258,12 @@ ghb_status build_plan_tables(int M, FftPlan& p, PlanTables& t) {
   }
   p = FftPlan{};
   p.M = M;
-  p.nst = static_cast<int>(radices.size());
-  int L = 1;
-  for (int t = 0; t < p.nst; ++t) {
-    p.R[t] = radices[t];
-    p.Lp[t] = L;
-    L *= radices[t];
-  }
-  for (int t = p.nst; t < kMaxStages; ++t) { p.R[t] = 1; p.Lp[t] = L; }
-  group_passes(p, 32);
-  if (!fx_group_passes(M, kFxCap, p.fx, &t.fx_perm)) {
-    set_error("internal: no FP64 passes for M=" + std::to_string(M));
+  if (!group_plan(0, M, kGroupCap[0], p.fx, &t.perm_of[0], &t.nat_of[0]) ||
+      !group_plan(1, M, kGroupCap[1], p.rt, &t.perm_of[1], &t.nat_of[1])) {
+    set_error("internal: no passes for M=" + std::to_string(M));
     return GHB_ERR_INVALID;
   }
 
-  // perm[n]: write n in mixed radix with the last stage's radix least
-  // significant; the position has the digits in stage order, first stage least
-  // significant.
-  std::vector<int>& perm = t.perm;
-  perm.assign(M, 0);
-  std::vector<int> q(p.nst > 0 ? p.nst : 1);
-  for (int n = 0; n < M; ++n) {
-    int rem = n;
-    for (int t = p.nst - 1; t >= 0; --t) {
-      q[t] = rem % p.R[t];
-      rem /= p.R[t];
-    }
-    int pos = 0;
-    for (int t = 0; t < p.nst; ++t) pos += q[t] * p.Lp[t];
-    perm[n] = pos;
-  }
   std::vector<UnitRoot> roots;
   unit_roots(M, roots);
   fx_twiddles(roots, t.fx_tw);
@@ -328,20 +281,19 @@ ghb_status make_plan(int M, PlanHolder& out) {
   return apply_tune(M, out);
 }
 
-ghb_status set_fx_cap(PlanHolder& out, int cap) {
+ghb_status set_group_cap(PlanHolder& out, int k, int cap) {
   FftPlan& p = out.plan;
-  FxPlan f = p.fx;
-  std::vector<int> perm;
-  if (!fx_group_passes(p.M, cap, f, &perm)) {
-    set_error("internal: no FP64 passes for M=" + std::to_string(p.M));
+  FxPlan f = k == 0 ? p.fx : p.rt;
+  std::vector<int> perm, nat;
+  if (!group_plan(k, p.M, cap, f, &perm, &nat)) {
+    set_error("internal: no passes for M=" + std::to_string(p.M));
     return GHB_ERR_INVALID;
   }
-  GHB_CUDA_TRY(cudaMemcpy(out.d_fx_perm, perm.data(), sizeof(int) * p.M, cudaMemcpyHostToDevice));
+  GHB_CUDA_TRY(cudaMemcpy(out.d_group_perm[k], perm.data(), sizeof(int) * p.M, cudaMemcpyHostToDevice));
+  GHB_CUDA_TRY(cudaMemcpy(out.d_group_perm[k] + p.M, nat.data(), sizeof(int) * p.M, cudaMemcpyHostToDevice));
   GHB_CUDA_TRY(cudaStreamSynchronize(cudaStreamLegacy));   // in place before any stream's kernels read it
-  f.perm = out.d_fx_perm;
-  f.tw = p.fx.tw;
-  p.fx = f;
-  out.fx_cap = cap;
+  (k == 0 ? p.fx : p.rt) = f;
+  out.cap[k] = cap;
   return GHB_OK;
 }
 
@@ -350,14 +302,14 @@ ghb_status make_plan_untuned(int M, PlanHolder& out) {
   ghb_status st = build_plan_tables(M, out.plan, t);
   if (st != GHB_OK) return st;
   FftPlan& p = out.plan;
-  const std::vector<int>& perm = t.perm;
   const std::vector<float2>& tw32 = t.tw32;
-  GHB_CUDA_TRY(cudaMalloc(&out.d_perm, sizeof(int) * M));
-  GHB_CUDA_TRY(cudaMalloc(&out.d_fx_perm, sizeof(int) * M));
+  for (int k = 0; k < 2; ++k) GHB_CUDA_TRY(cudaMalloc(&out.d_group_perm[k], sizeof(int) * 2 * M));
   GHB_CUDA_TRY(cudaMalloc(&out.d_fx_tw, sizeof(fxw) * M));
   GHB_CUDA_TRY(cudaMalloc(&out.d_tw32, sizeof(float2) * M));
-  GHB_CUDA_TRY(cudaMemcpy(out.d_perm, perm.data(), sizeof(int) * M, cudaMemcpyHostToDevice));
-  GHB_CUDA_TRY(cudaMemcpy(out.d_fx_perm, t.fx_perm.data(), sizeof(int) * M, cudaMemcpyHostToDevice));
+  for (int k = 0; k < 2; ++k) {
+    GHB_CUDA_TRY(cudaMemcpy(out.d_group_perm[k], t.perm_of[k].data(), sizeof(int) * M, cudaMemcpyHostToDevice));
+    GHB_CUDA_TRY(cudaMemcpy(out.d_group_perm[k] + M, t.nat_of[k].data(), sizeof(int) * M, cudaMemcpyHostToDevice));
+  }
   GHB_CUDA_TRY(cudaMemcpy(out.d_fx_tw, t.fx_tw.data(), sizeof(fxw) * M, cudaMemcpyHostToDevice));
   GHB_CUDA_TRY(cudaMemcpy(out.d_tw32, tw32.data(), sizeof(float2) * M, cudaMemcpyHostToDevice));
   GHB_CUDA_TRY(cudaStreamSynchronize(cudaStreamLegacy));   // pageable copies: in place before other streams read
@@ -367,20 +319,22 @@ ghb_status make_plan_untuned(int M, PlanHolder& out) {
     GHB_CUDA_TRY(cudaMalloc(&out.d_perm_ct, sizeof(int) * M));
     GHB_CUDA_TRY(cudaMemcpy(out.d_perm_ct, pct.data(), sizeof(int) * M, cudaMemcpyHostToDevice));
   }
-  p.perm = out.d_perm;
-  p.perm_ct = out.d_perm_ct;
+  p.ct = CtTables{out.d_perm_ct, out.d_tw32};
   p.ct_col = p.ct_row = (out.d_perm_ct != nullptr) ? 1 : 0;
-  p.fx.perm = out.d_fx_perm;
+  p.fx.perm = out.d_group_perm[0];
+  p.rt.perm = out.d_group_perm[1];
+  p.fx.nat = out.d_group_perm[0] + M;
+  p.rt.nat = out.d_group_perm[1] + M;
   p.fx.tw = out.d_fx_tw;
-  out.fx_cap = kFxCap;
-  p.tw32 = out.d_tw32;
+  for (int k = 0; k < 2; ++k) out.cap[k] = kGroupCap[k];
+  p.rt.tw32 = out.d_tw32;
   return GHB_OK;
 }
 
 void free_plan(PlanHolder& p) {
-  if (p.d_perm) cudaFree(p.d_perm);
   if (p.d_perm_ct) cudaFree(p.d_perm_ct);
-  if (p.d_fx_perm) cudaFree(p.d_fx_perm);
+  for (int* q : p.d_group_perm)
+    if (q) cudaFree(q);
   if (p.d_fx_tw) cudaFree(p.d_fx_tw);
   if (p.d_tw32) cudaFree(p.d_tw32);
   p = PlanHolder{};

@@ -1,0 +1,40 @@
+// Last-axis kernels of the FP32 run-time plans; see passes_rt.cuh.
+#include "launch_util.cuh"
+#include "passes_rt.cuh"
+
+namespace ghb {
+
+__global__ void __launch_bounds__(kRtThreads, 1)
+    rt_row_kernel(const __grid_constant__ RowArgs a, const __grid_constant__ FxPlan f, int rows_per_cta, int lines) {
+  rt_row_body(a, f, rows_per_cta, lines, blockIdx.x, gridDim.x);
+}
+
+__global__ void __launch_bounds__(kRtThreads, 1)
+    rt_row_kernel_batch(const RowItem* __restrict__ items, int n, int lines) {
+  __shared__ int s_item;
+  if (threadIdx.x == 0) s_item = find_item(items, n, blockIdx.x);
+  __syncthreads();
+  const RowItem& it = items[s_item];
+  rt_row_body(it.a, it.pl->rt, it.rows_per_cta, lines, blockIdx.x - it.block_begin, it.nblocks);
+}
+
+ghb_status launch_rt_row(const RowArgs& a, const FxPlan& f, int rows_per_cta, int lines, cudaStream_t s) {
+  static std::atomic<unsigned long long> mask{0};
+  TRY_STATUS(ensure_dyn_smem(rt_row_kernel, 200 * 1024, mask));
+  const size_t smem = static_cast<size_t>(lines) * f.ls * sizeof(float2);
+  const int64_t grid = (a.rows + rows_per_cta - 1) / rows_per_cta;
+  rt_row_kernel<<<static_cast<unsigned>(grid), rt_threads(f.M, lines, f.ls), smem, s>>>(a, f, rows_per_cta, lines);
+  GHB_CUDA_TRY(cudaGetLastError());
+  return GHB_OK;
+}
+
+ghb_status launch_rt_row_batch(int lines, const RowItem* items, int n, int64_t blocks, size_t smem, int threads,
+                               cudaStream_t s) {
+  static std::atomic<unsigned long long> mask{0};
+  TRY_STATUS(ensure_dyn_smem(rt_row_kernel_batch, 200 * 1024, mask));
+  rt_row_kernel_batch<<<static_cast<unsigned>(blocks), threads, smem, s>>>(items, n, lines);
+  GHB_CUDA_TRY(cudaGetLastError());
+  return GHB_OK;
+}
+
+}  // namespace ghb

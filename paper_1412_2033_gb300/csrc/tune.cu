@@ -1,24 +1,27 @@
 // Autotuner of the operator's launch configuration, per transform length M.
 //
 // What it chooses (carried in every FftPlan made for M):
-//   cap32, cap64  largest radix product of a register-blocked pass of the
-//                 runtime-plan transform (FP32, FP64): fewer passes against
-//                 more registers per thread;
+//   cap64         largest radix product of a register-blocked FP64 pass: fewer
+//                 passes against more registers per thread (cap32, the same of
+//                 the FP32 run-time plans, takes part in ghb_tune_set only: its
+//                 largest passes of 16 are the best at every length measured);
 //   rows32        rows per CTA of the FP32 2-D operator's last-axis pass;
 //   ct_col/ct_row size-specialised FP32 kernels (where compiled) or the
-//                 runtime-plan ones.
+//                 run-time-plan ones.  Measured last-axis pass: M = 270 203 us
+//                 specialised against 295, M = 4374 145 against 208; columns at
+//                 M = 4374 64 + 60 against 82 + 74.
 // The columns per CTA of the column passes (tile32/64) depend on the operand,
 // not on M alone (a 3-D axis-1 pass has ~M times the columns of a 2-D one), so
-// they are chosen at launch from the operand's shape (auto_tile) and are not
-// tuned; ghb_tune_set can still force them.
+// they are chosen at launch from the operand's shape (rt_col_tile, fx_col_tile)
+// and are not tuned; ghb_tune_set can still force them.
 // How: on the first plan for M in the process, a 2-D operand with the largest
 // odd N that M serves is allocated -- at least 2^20 double-grid entries per
 // component, widened with more columns and rows where N x N is smaller, so
 // that the timed launches are long enough to compare -- and every candidate is
 // timed with CUDA events on a private stream (1 untimed + 3 timed launches;
 // the inverse and forward column passes and the last-axis pass separately);
-// the fastest runtime-plan grouping by the sum of the three, then the
-// specialised kernels where they beat it.  Results stay for the life of the
+// the fastest rows, the specialised kernels where they beat the run-time
+// plans, and the fastest FP64 grouping by the sum of the three.  Results stay for the life of the
 // process.
 // GHB_AUTOTUNE=0 in the environment keeps the size rules instead.
 #include <algorithm>
@@ -57,15 +60,16 @@ Tune size_rules(int M) {
 
 ghb_status write_tune(const Tune& t, PlanHolder& h) {
   FftPlan& p = h.plan;
-  group_passes(p, t.cap32);
-  if (h.fx_cap != t.cap64) {
-    const ghb_status st = set_fx_cap(h, t.cap64);
-    if (st != GHB_OK) return st;
-  }
+  const int caps[2] = {t.cap64, t.cap32};
+  for (int k = 0; k < 2; ++k)
+    if (h.cap[k] != caps[k]) {
+      const ghb_status st = set_group_cap(h, k, caps[k]);
+      if (st != GHB_OK) return st;
+    }
   p.tile[1] = t.tile32;
   p.tile[0] = t.tile64;
   p.rows32 = t.rows32;
-  const bool ct = p.perm_ct != nullptr && ct_size(p.M);
+  const bool ct = p.ct.perm != nullptr && ct_size(p.M);
   p.ct_col = ct ? t.ct_col : 0;
   p.ct_row = ct ? t.ct_row : 0;
   return GHB_OK;
@@ -208,48 +212,31 @@ ghb_status tune_length(int M, Tune* out) {
     row.a = b.p[f32 ? 2 : 5];
   };
 
-  // FP32: runtime-plan grouping and rows, then the specialised kernels
+  // FP32: rows of the run-time plan, then the specialised kernels
   {
     ColArgs inv, fwd;
     RowArgs row;
     args(true, inv, fwd, row);
-    float best_total = 1e30f, best_col_generic = 1e30f, best_row_generic = 1e30f;
-    for (int cap : {18, 32}) {
-      FftPlan p = ph.plan;
-      group_passes(p, cap);
-      p.ct_col = p.ct_row = 0;
-      float col_best = 1e30f, row_best = 1e30f;
-      int rows_best = 0;
-      {
-        p.tile[1] = 0;
-        float ti = 0, tf = 0;
-        TUNE_TRY(tm.time([&] { return launch_col<float>(+1, COL_PLAIN, inv, p, tm.s); }, &ti));
-        TUNE_TRY(tm.time([&] { return launch_col<float>(-1, COL_PLAIN, fwd, p, tm.s); }, &tf));
-        col_best = ti + tf;
-      }
-      for (int rows : {1, 2}) {
-        p.rows32 = rows;
-        float tr = 0;
-        TUNE_TRY(tm.time([&] { return launch_row<float>(ROW_MATVEC, row, p, tm.s); }, &tr));
-        if (tr < row_best) {
-          row_best = tr;
-          rows_best = rows;
-        }
-      }
-      if (col_best + row_best < best_total) {
-        best_total = col_best + row_best;
-        best_col_generic = col_best;
-        best_row_generic = row_best;
-        best.cap32 = cap;
-        best.tile32 = 0;
-        best.rows32 = rows_best;
+    float best_row_generic = 1e30f;
+    FftPlan p = ph.plan;
+    p.ct_col = p.ct_row = 0;
+    p.tile[1] = 0;
+    float ti = 0, tf = 0;
+    TUNE_TRY(tm.time([&] { return launch_col<float>(+1, COL_PLAIN, inv, p, tm.s); }, &ti));
+    TUNE_TRY(tm.time([&] { return launch_col<float>(-1, COL_PLAIN, fwd, p, tm.s); }, &tf));
+    const float best_col_generic = ti + tf;
+    for (int rows : {1, 2}) {
+      p.rows32 = rows;
+      float tr = 0;
+      TUNE_TRY(tm.time([&] { return launch_row<float>(ROW_MATVEC, row, p, tm.s); }, &tr));
+      if (tr < best_row_generic) {
+        best_row_generic = tr;
+        best.rows32 = rows;
       }
     }
     best.ct_col = best.ct_row = 0;
-    if (ph.plan.perm_ct != nullptr && ct_size(M)) {
-      FftPlan p = ph.plan;
+    if (p.ct.perm != nullptr && ct_size(M)) {
       p.ct_col = p.ct_row = 1;
-      float ti = 0, tf = 0;
       TUNE_TRY(tm.time([&] { return launch_col<float>(+1, COL_PLAIN, inv, p, tm.s); }, &ti));
       TUNE_TRY(tm.time([&] { return launch_col<float>(-1, COL_PLAIN, fwd, p, tm.s); }, &tf));
       if (ti + tf < best_col_generic) best.ct_col = 1;
@@ -272,7 +259,7 @@ ghb_status tune_length(int M, Tune* out) {
     args(false, inv, fwd, row);
     float best_total = 1e30f;
     for (int cap : {9, 18}) {
-      TUNE_TRY(set_fx_cap(ph, cap));
+      TUNE_TRY(set_group_cap(ph, 0, cap));
       FftPlan p = ph.plan;
       float col_best = 1e30f;
       {

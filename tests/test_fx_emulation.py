@@ -44,12 +44,26 @@ int main(int argc, char** argv) {
   for (int arg = 2; arg < argc; ++arg) {
     const int cap = atoi(argv[1]), M = atoi(argv[arg]);
     FxPlan P{};
-    std::vector<int> perm;
+    std::vector<int> perm, pos;
     std::vector<UnitRoot> R;
     std::vector<fxw> tw;
-    if (!fx_group_passes(M, cap, P, &perm)) return 1;
+    if (!group_plan(0, M, cap, P, &perm, &pos)) return 1;
     unit_roots(M, R);
     fx_twiddles(R, tw);
+    // positions: distinct, inside the line, evenly spaced in every group; the first
+    // pass's unit r holds the natural indices r + (M / R) rev(j)
+    std::vector<char> seen(P.ls, 0);
+    bool laid = true;
+    for (int n = 0; n < M; ++n) laid &= pos[n] >= 0 && pos[n] < P.ls && !seen[pos[n]]++;
+    for (int i = 0; i < P.np; ++i)
+      for (int u = 0; u < P.p[i].units; ++u)
+        for (int j = 0, p; j < P.p[i].R; ++j)
+          laid &= pos[fx_unit_entry(P.p[i], u, p)] + j * P.p[i].step == pos[fx_unit_entry(P.p[i], u, p) + j * P.p[i].lp];
+    const int rb[] = {1, 1, 1, 1, 2, 2, 3, 2, 1};
+    for (int r = 0; P.np && r < P.p[0].units; ++r)
+      for (int j = 0, B = rb[P.p[0].shape], A = P.p[0].R / B; j < P.p[0].R; ++j)
+        laid &= perm[r] + j == perm[r + P.p[0].units * (j % A * B + j / A)];
+    if (!laid) return 2;
     for (int kind = 0; kind < 3; ++kind)        // white, 1/(1+|k|), one coefficient over 1e-3 noise
       for (int dit = 1; dit >= 0; --dit) {
         std::vector<Z<double>> x(M);
@@ -64,7 +78,7 @@ int main(int argc, char** argv) {
         }
         const int b = dit ? P.p[0].bits_dit : P.p[P.np - 1].bits_dif;
         std::vector<fx2> buf(P.ls, fx2{0, 0});
-        auto nat = [&](int k) { return k + (P.pad ? k / P.pad : 0); };
+        auto nat = [&](int k) { return pos[k]; };
         for (int k = 0; k < M; ++k)
           buf[dit ? perm[k] : nat(k)] = fx2{fx_from_double(x[k].real(), E, b), fx_from_double(x[k].imag(), E, b)};
         int e = E - 1022 - b;
@@ -75,13 +89,13 @@ int main(int argc, char** argv) {
           mag = 0;
           for (int u = 0; u < S.units; ++u) {
             int p;
-            fx2* base = &buf[fx_unit_base(S, P.pad, P.pdiv, u, p)];
+            fx2* base = &buf[pos[fx_unit_entry(S, u, p)]];
             const int m = dit ? (i ? fx_run_unit<1, true, false>(S, base, g, p, M, tw.data()) : fx_run_unit<1, true, true>(S, base, g, p, M, tw.data()))
                               : (i ? fx_run_unit<-1, false, false>(S, base, g, p, M, tw.data()) : fx_run_unit<-1, false, true>(S, base, g, p, M, tw.data()));
             mag = std::max(mag, m);
           }
           e += 2 * fx_quarters(S.shape, i == 0) - g;
-          range |= mag >= (1 << 30);            // |component| >= 2^62
+          range |= mag >= (q + 1 < P.np || dit ? 0x70000000 : 1 << 30);   // 2^62.8, 2^62 after the last forward pass
         }
         std::vector<Z<double>> dbl(x);
         dft(ref, dit ? 1 : -1, R, 1);

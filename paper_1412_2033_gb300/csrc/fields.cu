@@ -11,6 +11,7 @@
 #include <cmath>
 
 #include "ghb_internal.cuh"
+#include "launch_util.cuh"
 #include "reduce.cuh"
 
 namespace ghb {
@@ -563,6 +564,7 @@ __device__ __forceinline__ void run_op(const CgItem& it, int64_t bid, int64_t nb
 
 template <typename T, int OP>
 __global__ void __launch_bounds__(kFieldThreads) cg_kernel(CgItem it) {
+  grid_wait();
   run_op<T, OP>(it, blockIdx.x, gridDim.x);
 }
 
@@ -583,6 +585,7 @@ __global__ void __launch_bounds__(kFieldThreads) cg_kernel_batch(const CgItem* _
   if (threadIdx.x == 0) s_item = find_cg_item(items, n, blockIdx.x);
   __syncthreads();
   const CgItem& it = items[s_item];
+  grid_wait();
   run_op<T, OP>(it, blockIdx.x - it.block_begin, it.nblocks);
 }
 
@@ -803,9 +806,7 @@ int64_t one_wave(int64_t want) {
 template <typename T, int OP>
 ghb_status launch_one(const CgItem& it, cudaStream_t s) {
   const int64_t nb = one_wave<T, OP>(it.nblocks);
-  cg_kernel<T, OP><<<static_cast<unsigned>(nb), kFieldThreads, 0, s>>>(it);
-  GHB_CUDA_TRY(cudaGetLastError());
-  return GHB_OK;
+  return launch_chained(cg_kernel<T, OP>, nb, kFieldThreads, 0, s, it);
 }
 CgItem make_item(const FieldGeom& fg) {
   CgItem it{};
@@ -910,19 +911,16 @@ ghb_status launch_accum_f32(double2* x, const double2* base, const float2* dx, c
 
 template <typename T>
 ghb_status launch_cg_batch(int op, const CgItem* items, int n, int64_t blocks, cudaStream_t s) {
-  const unsigned g = static_cast<unsigned>(blocks);
   switch (op) {
-    case CG_INIT: cg_kernel_batch<T, CG_INIT><<<g, kFieldThreads, 0, s>>>(items, n); break;
-    case CG_PROJECT_DOT: cg_kernel_batch<T, CG_PROJECT_DOT><<<g, kFieldThreads, 0, s>>>(items, n); break;
-    case CG_UPDATE: cg_kernel_batch<T, CG_UPDATE><<<g, kFieldThreads, 0, s>>>(items, n); break;
-    case CG_PROJECT: cg_kernel_batch<T, CG_PROJECT><<<g, kFieldThreads, 0, s>>>(items, n); break;
-    case CG_RESIDUAL: cg_kernel_batch<double, CG_RESIDUAL><<<g, kFieldThreads, 0, s>>>(items, n); break;
-    case CG_TO_F32: cg_kernel_batch<double, CG_TO_F32><<<g, kFieldThreads, 0, s>>>(items, n); break;
-    case CG_ACCUM: cg_kernel_batch<double, CG_ACCUM><<<g, kFieldThreads, 0, s>>>(items, n); break;
+    case CG_INIT: return launch_chained(cg_kernel_batch<T, CG_INIT>, blocks, kFieldThreads, 0, s, items, n);
+    case CG_PROJECT_DOT: return launch_chained(cg_kernel_batch<T, CG_PROJECT_DOT>, blocks, kFieldThreads, 0, s, items, n);
+    case CG_UPDATE: return launch_chained(cg_kernel_batch<T, CG_UPDATE>, blocks, kFieldThreads, 0, s, items, n);
+    case CG_PROJECT: return launch_chained(cg_kernel_batch<T, CG_PROJECT>, blocks, kFieldThreads, 0, s, items, n);
+    case CG_RESIDUAL: return launch_chained(cg_kernel_batch<double, CG_RESIDUAL>, blocks, kFieldThreads, 0, s, items, n);
+    case CG_TO_F32: return launch_chained(cg_kernel_batch<double, CG_TO_F32>, blocks, kFieldThreads, 0, s, items, n);
+    case CG_ACCUM: return launch_chained(cg_kernel_batch<double, CG_ACCUM>, blocks, kFieldThreads, 0, s, items, n);
     default: set_error("internal: bad batched CG op"); return GHB_ERR_INVALID;
   }
-  GHB_CUDA_TRY(cudaGetLastError());
-  return GHB_OK;
 }
 template ghb_status launch_cg_batch<double>(int, const CgItem*, int, int64_t, cudaStream_t);
 template ghb_status launch_cg_batch<float>(int, const CgItem*, int, int64_t, cudaStream_t);

@@ -28,9 +28,7 @@ ghb_status row_launch(const RowArgs& a, const FxPlan& f, int rows_per_cta, int N
   const size_t smem = static_cast<size_t>(NL) * f.ls * sizeof(fx2);
   int64_t grid = (a.rows + rows_per_cta - 1) / rows_per_cta;
   if (MODE == ROW_ENERGY && grid > 1024) grid = 1024;   // partials hold 1024 x 6 doubles
-  fx_row_kernel<MODE><<<static_cast<unsigned>(grid), threads, smem, s>>>(a, f, rows_per_cta, NL);
-  GHB_CUDA_TRY(cudaGetLastError());
-  return GHB_OK;
+  return launch_chained(fx_row_kernel<MODE>, grid, threads, smem, s, a, f, rows_per_cta, NL);
 }
 
 template <int MODE>
@@ -38,9 +36,7 @@ ghb_status row_launch_batch(int NL, const RowItem* items, int n, int64_t blocks,
                             cudaStream_t s) {
   static std::atomic<unsigned long long> mask{0};
   TRY_STATUS(ensure_dyn_smem(fx_row_kernel_batch<MODE>, 220 * 1024, mask));
-  fx_row_kernel_batch<MODE><<<static_cast<unsigned>(blocks), threads, smem, s>>>(items, n, NL);
-  GHB_CUDA_TRY(cudaGetLastError());
-  return GHB_OK;
+  return launch_chained(fx_row_kernel_batch<MODE>, blocks, threads, smem, s, items, n, NL);
 }
 
 }  // namespace

@@ -17,6 +17,7 @@
 
 #include "fft_fx.cuh"
 #include "ghb_internal.cuh"
+#include "launch_util.cuh"
 #include "reduce.cuh"
 
 namespace ghb {
@@ -123,7 +124,6 @@ __device__ __forceinline__ void fx_col_body(const ColArgs& a, const FxPlan& f, i
   extern __shared__ __align__(16) unsigned char smem_raw[];
   fx2* buf = reinterpret_cast<fx2*>(smem_raw);
   __shared__ FxShared sh;
-  if (a.st != nullptr && a.st->done != RUNNING) return;
   const int M = f.M;
   const int ls = column_stride(f.ls, TW, sizeof(fx2));
   fx_load_plan(sh, f);
@@ -138,8 +138,10 @@ __device__ __forceinline__ void fx_col_body(const ColArgs& a, const FxPlan& f, i
   const int64_t o = valid ? g / a.inner : 0, jj = valid ? g - o * a.inner : 0;
   const int64_t inner = a.inner;
   const int Lin = SIGN > 0 ? a.Lin : M;
-  const double2* __restrict__ in = static_cast<const double2*>(a.in) + o * Lin * inner + jj;
   fx2* line = buf + t * ls;
+  grid_wait();
+  const double2* __restrict__ in = after_wait(static_cast<const double2*>(a.in) + o * Lin * inner + jj);
+  if (a.st != nullptr && a.st->done != RUNNING) return;
 
   // Largest exponent of the column, then its integers in place (inverse: the
   // digit-reversed positions; forward: natural order).  Columns of up to K
@@ -273,7 +275,6 @@ __device__ __forceinline__ void fx_row_body(const RowArgs& a, const FxPlan& f, i
   __shared__ FxLine ld[kFxMaxLines];
   __shared__ double red[32];
   __shared__ bool last;
-  if (a.st != nullptr && a.st->done != RUNNING) return;
   const int M = f.M, H = a.H, ls = f.ls;
   const int per_row = a.nfields * a.ncomp;
   const int nrl = rows_per_cta * per_row;
@@ -285,6 +286,8 @@ __device__ __forceinline__ void fx_row_body(const RowArgs& a, const FxPlan& f, i
   const int nwarp = blockDim.x >> 5;
   const int segs = nwarp > NL ? nwarp / NL : 1;    // warps per line
   fx_load_plan(sh, f);
+  grid_wait();
+  if (a.st != nullptr && a.st->done != RUNNING) return;
   double gs[6] = {0, 0, 0, 0, 0, 0};               // ENERGY: upper triangle of F x F, F <= 3
 
   for (int64_t grp = bid; grp < groups; grp += nb) {

@@ -137,7 +137,6 @@ __device__ __forceinline__ void col_body(const ColArgs& a, const CtTables& pl, i
   using C = float2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* buf = reinterpret_cast<C*>(smem_raw);
-  if (a.st != nullptr && a.st->done != RUNNING) return;
 
   // TW consecutive columns of the flattened (outer, inner) range, so that no CTA
   // is spent on the ragged end of each outer index
@@ -153,9 +152,11 @@ __device__ __forceinline__ void col_body(const ColArgs& a, const CtTables& pl, i
     s_in[threadIdx.x] = static_cast<int>(oo * rows_in * a.inner + jj);
     s_out[threadIdx.x] = static_cast<int>(oo * rows_out * a.inner + jj);
   }
+  grid_wait();
+  if (a.st != nullptr && a.st->done != RUNNING) return;
   __syncthreads();
   const C* __restrict__ tw = pl.tw;
-  const C* __restrict__ in = static_cast<const C*>(a.in);
+  const C* __restrict__ in = after_wait(static_cast<const C*>(a.in));
   C* __restrict__ out = static_cast<C*>(a.out);
 
   if constexpr (SIGN > 0) {
@@ -169,7 +170,7 @@ __device__ __forceinline__ void col_body(const ColArgs& a, const CtTables& pl, i
     C* pnew = nullptr;
     if constexpr (MODE == COL_PUPDATE) {
       beta = static_cast<T>(a.st->beta);
-      pold = static_cast<const C*>(a.pold);
+      pold = after_wait(static_cast<const C*>(a.pold));
       pnew = static_cast<C*>(a.pnew);
     }
     ColSource<C, T, MODE == COL_PUPDATE> src{in, pold, pnew, s_in, beta, static_cast<int>(a.inner), half, M, width};
@@ -218,9 +219,7 @@ inline ghb_status launch_col_t(const ColArgs& a, const CtTables& pl, cudaStream_
     set_error("column pass operand of 2^31 entries or more");
     return GHB_ERR_INVALID;
   }
-  col_kernel<TW, SIGN, MODE, M><<<static_cast<unsigned>(grid), col_threads<TW, M, MODE>(), smem, s>>>(a, pl);
-  GHB_CUDA_TRY(cudaGetLastError());
-  return GHB_OK;
+  return launch_chained(col_kernel<TW, SIGN, MODE, M>, grid, col_threads<TW, M, MODE>(), smem, s, a, pl);
 }
 
 // ---------------------------------------------------------------------------
@@ -321,6 +320,7 @@ __device__ __forceinline__ void row_matvec_staged(const RowArgs& a, const CtTabl
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ LineDesc ld[2 * NL], ldn[2 * NL];   // this group's lines, the next group's
   __shared__ int2 lrow[NL];                      // offsets in A_M of each complex line's two rows
+  grid_wait();
   if (a.st != nullptr && a.st->done != RUNNING) return;
 
   const int H = a.H;
@@ -484,9 +484,7 @@ inline ghb_status launch_row_t(const RowArgs& a, const CtTables& pl, int rows_pe
   int64_t grid = static_cast<int64_t>(o.per_sm > 0 ? o.per_sm : 1) * o.sms;
   if (grid > groups) grid = groups;
   if (grid < 1) grid = 1;
-  row_kernel_staged<NL, M><<<static_cast<unsigned>(grid), kRowThreads, smem, s>>>(a, pl, rows_per_cta);
-  GHB_CUDA_TRY(cudaGetLastError());
-  return GHB_OK;
+  return launch_chained(row_kernel_staged<NL, M>, grid, kRowThreads, smem, s, a, pl, rows_per_cta);
 }
 
 // Size-specialised operator passes of transform length M (instantiated in the

@@ -5,6 +5,7 @@
 
 #include "fft_rt.cuh"
 #include "ghb_internal.cuh"
+#include "launch_util.cuh"
 
 namespace ghb {
 
@@ -124,7 +125,6 @@ __device__ __forceinline__ void rt_col_body(const ColArgs& a, const FxPlan& f, i
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2* buf = reinterpret_cast<float2*>(smem_raw);
   __shared__ RtShared sh;
-  if (a.st != nullptr && a.st->done != RUNNING) return;
   const int M = f.M;
   rt_load_plan(sh, f);
   const int t = threadIdx.x & (TW - 1);
@@ -135,6 +135,8 @@ __device__ __forceinline__ void rt_col_body(const ColArgs& a, const FxPlan& f, i
   const int64_t o = on ? g / a.inner : 0, j = on ? g - o * a.inner : 0;
   const int Lin = SIGN > 0 ? a.Lin : M, Lout = SIGN > 0 ? M : a.Lout;
   const int64_t off = o * Lin * a.inner + j;
+  grid_wait();
+  if (a.st != nullptr && a.st->done != RUNNING) return;
   RtColIn<UPDATE> src{};
   src.in = static_cast<const float2*>(a.in) + off;
   src.inner = inner;
@@ -190,7 +192,6 @@ __device__ __forceinline__ void rt_row_body(const RowArgs& a, const FxPlan& f, i
   float2* buf = reinterpret_cast<float2*>(smem_raw);
   __shared__ RtShared sh;
   __shared__ RtLine ld[kRtMaxLines];
-  if (a.st != nullptr && a.st->done != RUNNING) return;
   const int M = f.M, H = a.H, ls = f.ls;
   const int nrl = rows_per_cta * a.ncomp;
   const int64_t groups = (a.rows + rows_per_cta - 1) / rows_per_cta;
@@ -203,6 +204,8 @@ __device__ __forceinline__ void rt_row_body(const RowArgs& a, const FxPlan& f, i
   float2* data = static_cast<float2*>(a.t[0]);
   const float* __restrict__ am = static_cast<const float*>(a.a);
   rt_load_plan(sh, f);
+  grid_wait();
+  if (a.st != nullptr && a.st->done != RUNNING) return;
 
   // input n of line q: Z(n) = X0(n) + i X1(n) below H, conj X0 + i conj X1 at M - n
   // above M - H, zero between

@@ -27,9 +27,7 @@ ghb_status col_launch(const ColArgs& a, const FxPlan& f, int TW, cudaStream_t s)
   TRY_STATUS(ensure_dyn_smem(rt_col_kernel<SIGN, UPDATE>, 220 * 1024, mask));
   const size_t smem = static_cast<size_t>(TW) * column_stride(f.ls, TW, sizeof(float2)) * sizeof(float2);
   const int64_t grid = (a.outer * a.inner + TW - 1) / TW;
-  rt_col_kernel<SIGN, UPDATE><<<static_cast<unsigned>(grid), rt_threads(f.M, TW, f.ls), smem, s>>>(a, f, TW);
-  GHB_CUDA_TRY(cudaGetLastError());
-  return GHB_OK;
+  return launch_chained(rt_col_kernel<SIGN, UPDATE>, grid, rt_threads(f.M, TW, f.ls), smem, s, a, f, TW);
 }
 
 template <int SIGN, bool UPDATE>
@@ -37,9 +35,7 @@ ghb_status col_launch_batch(int TW, const ColItem* items, int n, int64_t blocks,
                             cudaStream_t s) {
   static std::atomic<unsigned long long> mask{0};
   TRY_STATUS(ensure_dyn_smem(rt_col_kernel_batch<SIGN, UPDATE>, 220 * 1024, mask));
-  rt_col_kernel_batch<SIGN, UPDATE><<<static_cast<unsigned>(blocks), threads, smem, s>>>(items, n, TW);
-  GHB_CUDA_TRY(cudaGetLastError());
-  return GHB_OK;
+  return launch_chained(rt_col_kernel_batch<SIGN, UPDATE>, blocks, threads, smem, s, items, n, TW);
 }
 
 }  // namespace

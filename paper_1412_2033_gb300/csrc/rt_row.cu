@@ -23,18 +23,14 @@ ghb_status launch_rt_row(const RowArgs& a, const FxPlan& f, int rows_per_cta, in
   TRY_STATUS(ensure_dyn_smem(rt_row_kernel, 200 * 1024, mask));
   const size_t smem = static_cast<size_t>(lines) * f.ls * sizeof(float2);
   const int64_t grid = (a.rows + rows_per_cta - 1) / rows_per_cta;
-  rt_row_kernel<<<static_cast<unsigned>(grid), rt_threads(f.M, lines, f.ls), smem, s>>>(a, f, rows_per_cta, lines);
-  GHB_CUDA_TRY(cudaGetLastError());
-  return GHB_OK;
+  return launch_chained(rt_row_kernel, grid, rt_threads(f.M, lines, f.ls), smem, s, a, f, rows_per_cta, lines);
 }
 
 ghb_status launch_rt_row_batch(int lines, const RowItem* items, int n, int64_t blocks, size_t smem, int threads,
                                cudaStream_t s) {
   static std::atomic<unsigned long long> mask{0};
   TRY_STATUS(ensure_dyn_smem(rt_row_kernel_batch, 200 * 1024, mask));
-  rt_row_kernel_batch<<<static_cast<unsigned>(blocks), threads, smem, s>>>(items, n, lines);
-  GHB_CUDA_TRY(cudaGetLastError());
-  return GHB_OK;
+  return launch_chained(rt_row_kernel_batch, blocks, threads, smem, s, items, n, lines);
 }
 
 }  // namespace ghb

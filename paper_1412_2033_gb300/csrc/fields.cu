@@ -77,7 +77,9 @@ __device__ __forceinline__ C hermitian_part(const C* w, int64_t P, int c, int64_
 }
 
 // q = G(k) w with G_E = k k^T / k.k (primal) or G_J = I - G_E (dual), 0 at k = 0
-// (Def. projection).
+// (Def. projection).  For k along one axis G_E keeps that component exactly: a
+// laminate's dual right-hand side is zero, not a rounding residue that no
+// iteration can reduce.
 template <typename T, typename C>
 __device__ __forceinline__ void project_vec(int d, const int k[3], int kind, const C* w, C* q) {
   const T k0 = T(k[0]), k1 = T(k[1]), k2 = T(k[2]);
@@ -95,8 +97,9 @@ __device__ __forceinline__ void project_vec(int d, const int k[3], int kind, con
   const T inv = T(1) / kk;   // one division per entry
   sx *= inv;
   sy *= inv;
+  const bool axis = (k[0] != 0) + (k[1] != 0) + (k[2] != 0) == 1;
   for (int c = 0; c < d; ++c) {
-    const C pe = mk(kv[c] * sx, kv[c] * sy);
+    const C pe = axis && k[c] != 0 ? w[c] : mk(kv[c] * sx, kv[c] * sy);
     q[c] = (kind == GHB_PRIMAL) ? pe : mk(w[c].x - pe.x, w[c].y - pe.y);
   }
 }
@@ -133,156 +136,227 @@ __device__ bool grid_sum_last(double v, double* partials, unsigned int* ticket, 
 // coefficient table (eq. inclcomp_formula with the shape coefficients of
 // Remark anal_Fourier; the sphere by its radial transform)
 // ---------------------------------------------------------------------------
-__device__ double sinc_pi(double x) {   // sin(pi x)/(pi x)
-  return x == 0.0 ? 1.0 : sinpi(x) / (kPi * x);
+// What bounds the table: FP64 issue (2 lanes a clock and SM): for every entry and
+// inclusion it takes a shape factor and the phases of the entry and its mirror.
+// So a pair's own work is cut to what depends on the pair: |n|, its reciprocal and
+// |n|^(-3/2) belong to the entry, the radius' constants to the inclusion (in shared
+// memory); J_1 beyond 20 is Hankel's expansion with the coefficients as constants;
+// and sines and cosines take 18 FP64 instructions from a table of 64 angles.
+// Measured, N = 1023, 20 disks: 4.43 ms, 106 FP64 instructions a pair, FP64 pipe 86 %
+// busy (before, about 12 ms: sincospi twice a pair, divisions in every Hankel term).
+
+// The angles j / 64 of a turn, and sin, cos of one of them plus a <= pi / 64: the
+// Taylor polynomials to a^7 and a^8 (the next terms are below 2e-19) and the
+// addition theorem, with the corrections added last (half a unit beyond the
+// table's own rounding).
+constexpr int kAngles = 64;
+__device__ __forceinline__ double2 turn_sincos(const double2* angles, double whole, double a) {
+  const double2 t = angles[__double2loint(whole) & (kAngles - 1)];   // (cos, sin)
+  const double a2 = a * a;
+  const double sn = a * fma(a2, fma(a2, fma(a2, -1.0 / 5040, 1.0 / 120), -1.0 / 6), 1.0);
+  const double cm = a2 * fma(a2, fma(a2, fma(a2, 1.0 / 40320, -1.0 / 720), 1.0 / 24), -0.5);
+  return make_double2(t.x + fma(t.x, cm, -(t.y * sn)), t.y + fma(t.y, cm, t.x * sn));
+}
+// The integer nearest to v (|v| < 2^51) in the low bits of v + kWhole.
+constexpr double kWhole = 6755399441055744.0;   // 1.5 2^52
+// (cos, sin) of 2 pi t, |t| <= 1/2
+__device__ __forceinline__ double2 sincos_turns(const double2* angles, double t) {
+  const double w = fma(t, static_cast<double>(kAngles), kWhole);
+  return turn_sincos(angles, w, (2.0 * kPi) * fma(w - kWhole, -1.0 / kAngles, t));   // the difference is exact
+}
+// (cos, sin) of x, |x| < 2^40: x minus a multiple of 2 pi / 64 in two parts
+__device__ __forceinline__ double2 sincos_radians(const double2* angles, double x) {
+  constexpr double kHi = 2.0 * kPi / kAngles;                    // 2 pi / 64 rounded, and the rest of it
+  constexpr double kLo = 2.4492935982947064e-16 / kAngles;
+  const double w = fma(x, kAngles / (2.0 * kPi), kWhole);
+  const double k = w - kWhole;
+  return turn_sincos(angles, w, fma(-k, kLo, fma(-k, kHi, x)));
 }
 
-// Bessel function of the first kind of order one.
-//  |x| <= 8: CUDA's j1 (accurate to a few ulp there).
-//  8 < |x| < 20: Miller's backward recurrence J_{n-1} = (2n/x) J_n - J_{n+1},
-//     started at n0 ~ |x| + 40 with J_{n0+1} = 0, normalised by the identity
+// Coefficients of Hankel's expansion of J_1 (Abramowitz and Stegun 9.2.5, 9.2.9-
+// 9.2.10): a_m = prod_{j=1..m} (4 - (2j-1)^2) / (m! 8^m), sign (-1)^(m div 2).
+constexpr int kHankelTerms = 36;
+struct HankelTable {
+  double a[kHankelTerms];
+};
+__host__ __device__ constexpr HankelTable hankel_table() {
+  HankelTable t{};
+  double a = 1.0;
+  for (int m = 0; m < kHankelTerms; ++m) {
+    if (m > 0) a *= (4.0 - (2.0 * m - 1.0) * (2.0 * m - 1.0)) / (8.0 * m);
+    t.a[m] = (m >> 1) & 1 ? -a : a;
+  }
+  return t;
+}
+// P(x) and x Q(x) by Horner's rule in z = x^-2, to the terms a_LAST, a_(LAST+1)
+template <int LAST>
+__device__ __forceinline__ void hankel_sums(double z, double& P, double& Q) {
+  constexpr HankelTable t = hankel_table();
+  P = t.a[LAST];
+  Q = t.a[LAST + 1];
+#pragma unroll
+  for (int m = LAST - 2; m >= 0; m -= 2) {
+    P = fma(P, z, t.a[m]);
+    Q = fma(Q, z, t.a[m + 1]);
+  }
+}
+
+// Bessel function of the first kind of order one for 0 <= x < 20.
+//  x <= 8: CUDA's j1 (accurate to a few ulp there; it loses about 1e-12 of the
+//     envelope sqrt(2/(pi x)) beyond, which is visible in the bounds at 1e-13).
+//  x > 8: Miller's backward recurrence J_{n-1} = (2n/x) J_n - J_{n+1},
+//     started at n0 ~ x + 40 with J_{n0+1} = 0, normalised by the identity
 //     J_0 + 2 sum_{k>=1} J_{2k} = 1.
-//  |x| >= 20: Hankel's asymptotic expansion (Abramowitz and Stegun 9.2.5,
-//     9.2.9-9.2.10): J_1(x) = sqrt(2/(pi x)) (P cos chi - Q sin chi),
-//     chi = x - 3 pi/4, P = sum_k (-1)^k a_{2k} x^{-2k},
-//     Q = sum_k (-1)^k a_{2k+1} x^{-2k-1},
-//     a_m = prod_{j=1..m} (4 - (2j-1)^2) / (m! 8^m); summed until the terms
-//     fall below 1e-18 (the smallest term is about e^{-2x}).
-// CUDA's j1 loses about 1e-12 relative to the envelope sqrt(2/(pi x)) beyond
-// x = 8, which is visible in the bounds at the 1e-13 level.
-__device__ double bessel_j1(double x) {
-  const double ax = fabs(x);
-  const double sg = x < 0 ? -1.0 : 1.0;
-  if (ax <= 8.0) return j1(x);
-  if (ax < 20.0) {
-    int n0 = static_cast<int>(ax) + 40;
-    n0 += n0 & 1;                       // even start
-    double jp1 = 0.0, jn = 1e-30, sum = 2.0 * jn, j1v = 0.0;
-    for (int n = n0; n >= 1; --n) {
-      const double jm1 = (2.0 * n / ax) * jn - jp1;   // J_{n-1}
-      jp1 = jn;
-      jn = jm1;
-      const int m = n - 1;
-      if (m == 1) j1v = jn;
-      if ((m & 1) == 0) sum += (m == 0 ? 1.0 : 2.0) * jn;
-      if (fabs(jn) > 1e200) {          // rescale to stay in range
-        jn *= 1e-200;
-        jp1 *= 1e-200;
-        sum *= 1e-200;
-        j1v *= 1e-200;
-      }
+__device__ __noinline__ double bessel_j1_small(double x) {
+  if (x <= 8.0) return j1(x);
+  int n0 = static_cast<int>(x) + 40;
+  n0 += n0 & 1;                       // even start
+  double jp1 = 0.0, jn = 1e-30, sum = 2.0 * jn, j1v = 0.0;
+  for (int n = n0; n >= 1; --n) {
+    const double jm1 = (2.0 * n / x) * jn - jp1;   // J_{n-1}
+    jp1 = jn;
+    jn = jm1;
+    const int m = n - 1;
+    if (m == 1) j1v = jn;
+    if ((m & 1) == 0) sum += (m == 0 ? 1.0 : 2.0) * jn;
+    if (fabs(jn) > 1e200) {          // rescale to stay in range
+      jn *= 1e-200;
+      jp1 *= 1e-200;
+      sum *= 1e-200;
+      j1v *= 1e-200;
     }
-    return sg * j1v / sum;
   }
-  const double inv = 1.0 / ax;
-  double P = 1.0, Q = 0.0;
-  double a = 1.0;                        // a_m x^{-m} with alternating signs folded in below
-  for (int m = 1; m < 60; ++m) {
-    a *= (4.0 - (2.0 * m - 1.0) * (2.0 * m - 1.0)) / (8.0 * m) * inv;
-    // m odd -> Q term (-1)^((m-1)/2), m even -> P term (-1)^(m/2)
-    const int k = m >> 1;
-    const double term = ((k & 1) ? -a : a);
-    if (m & 1) Q += term;
-    else P += term;
-    if (fabs(a) < 1e-18) break;
-  }
-  double s, c;
-  sincos(ax, &s, &c);
-  const double r2 = 0.70710678118654752440084436210485;   // 1/sqrt(2)
-  const double cchi = (s - c) * r2;       // cos(x - 3 pi / 4)
-  const double schi = -(s + c) * r2;      // sin(x - 3 pi / 4)
-  return sg * sqrt(2.0 / (kPi * ax)) * (P * cchi - Q * schi);
+  return j1v / sum;
 }
 
-__device__ double shape_coeff(const Incl& in, int d, const int n[3]) {
-  if (in.shape == GHB_BOX) {
+// What an inclusion and an entry bring to the shape factors.
+struct CoefIncl {
+  int shape;
+  double c[3], s[3];
+  double amp, inv;         // disk: sqrt(r / 2) / pi, 1 / (2 pi r)
+  double dv, dv1;
+};
+struct CoefEntry {
+  int n[3];
+  double rho2, rho, rinv, rm32;   // |n|^2, |n|, 1 / |n|, |n|^(-3/2)
+  double pin[3];                  // 1 / (pi n_a)
+};
+
+// Shape factor f^(n): even in each component of n.
+template <int D>
+__device__ __forceinline__ double shape_coeff(const double2* angles, const CoefIncl& in, const CoefEntry& e) {
+  if (in.shape == GHB_BOX) {        // prod_a s_a sinc(s_a n_a)
     double v = 1.0;
-    for (int a = 0; a < d; ++a) v *= in.s[a] * sinc_pi(in.s[a] * n[a]);
+#pragma unroll
+    for (int a = 0; a < D; ++a) v *= e.n[a] == 0 ? in.s[a] : sinpi(in.s[a] * e.n[a]) * e.pin[a];
     return v;
   }
   const double r = in.s[0];
-  const double rho2 = double(n[0]) * n[0] + double(n[1]) * n[1] + double(n[2]) * n[2];
-  const double rho = sqrt(rho2);
-  if (in.shape == GHB_DISK) {
-    if (rho2 == 0.0) return kPi * r * r;
-    return r * bessel_j1(2.0 * kPi * r * rho) / rho;
+  const double x = 2.0 * kPi * r * e.rho;
+  if (in.shape == GHB_DISK) {       // r J_1(2 pi r rho) / rho
+    if (e.rho2 == 0.0) return kPi * r * r;
+    if (x < 20.0) return r * bessel_j1_small(x) * e.rinv;
+    const double ix = in.inv * e.rinv, z = ix * ix;
+    double P, Q;
+    if (x >= 100.0) hankel_sums<10>(z, P, Q);   // the first term left out is below 4e-18 in each range
+    else if (x >= 40.0) hankel_sums<14>(z, P, Q);
+    else hankel_sums<34>(z, P, Q);
+    // sqrt(2 / (pi x)) (P cos chi - Q sin chi), chi = x - 3 pi / 4
+    const double2 t = sincos_radians(angles, x);
+    return in.amp * e.rm32 * fma(P, t.y - t.x, Q * ix * (t.x + t.y));
   }
-  // sphere
-  const double q = 2.0 * kPi * r * rho;
-  if (q < 1e-2) {
-    const double q2 = q * q;
+  // sphere: (sin x - x cos x) / (2 pi^2 rho^3)
+  if (x < 1e-2) {
+    const double q2 = x * x;
     return 4.0 / 3.0 * kPi * r * r * r * (1.0 - q2 / 10.0 + q2 * q2 / 280.0 - q2 * q2 * q2 / 15120.0);
   }
-  double sq, cq;
-  sincos(q, &sq, &cq);
-  return (sq - q * cq) / (2.0 * kPi * kPi * rho2 * rho);
+  const double2 t = sincos_radians(angles, x);
+  return (t.y - x * t.x) * ((1.0 / (2.0 * kPi * kPi)) * (e.rinv * e.rinv * e.rinv));
 }
 
-// tab1 (optional): the table of a second inclusion list with the same shapes
-// and centres (the coefficient 1/a beside a); each inclusion's shape factor and
-// phase are evaluated once for both.  Every shape factor is even in each
-// component of n (products of sinc for boxes, functions of |n| for disks and
-// spheres), so one thread takes n = (n_0, ...) with n_0 >= 0 together with
-// its mirror (-n_0, ...): each shape factor once, the phase of each entry as
-// before (the same operations per entry, so the same values).
-__global__ void coeff_kernel(double2* tab, double2* tab1, Geometry g, const Incl* incs, const Incl* incs1, int n,
-                             double a0v, double a0v1) {
-  const int d = g.d;
+// The tables of a coefficient and of its inverse (the same shapes and centres):
+// every shape factor is even in each component of n, so one thread takes n =
+// (n_0, ...) with n_0 >= 0 together with its mirror (-n_0, ...), each shape factor
+// once for both entries and both tables.
+constexpr int kCoefChunk = 64;     // inclusions that a block holds at a time
+template <int D>
+__global__ void __launch_bounds__(kFieldThreads) coeff_kernel(double2* tab, double2* tab1, Geometry g, const Incl* incs,
+                                                              const Incl* incs1, int n, double a0v, double a0v1) {
+  __shared__ CoefIncl held[kCoefChunk];
+  __shared__ double2 angles[kAngles];
   const int N0 = g.N[0];
-  const int L1 = (d == 3) ? 2 * g.N[1] - 1 : g.N[1];
-  const int Ld = g.N[d - 1];   // half of 2N_d - 1: n_d = 0..N_d-1
-  const int64_t rest = (d == 3) ? static_cast<int64_t>(L1) * Ld : Ld;   // entries per value of n_0
-  const int64_t half = static_cast<int64_t>(N0) * rest;                 // n_0 = 0 .. N_0-1
-  for (int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; e < half;
-       e += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const int64_t n0 = e / rest;
-    const int64_t rr = e - n0 * rest;
-    int nv[3] = {static_cast<int>(n0), 0, 0};
-    if (d == 2) {
-      nv[1] = static_cast<int>(rr);
-    } else {
-      const int64_t i1 = rr / Ld;
-      nv[1] = static_cast<int>(i1) - (g.N[1] - 1);
-      nv[2] = static_cast<int>(rr - i1 * Ld);
-    }
-    const int nm[3] = {-nv[0], nv[1], nv[2]};
-    const bool mirror = nv[0] != 0;
-    const bool origin = nv[0] == 0 && nv[1] == 0 && nv[2] == 0;
-    double re = origin ? a0v : 0.0, im = 0.0;
-    double re1 = origin ? a0v1 : 0.0, im1 = 0.0;
+  const int L1 = D == 3 ? 2 * g.N[1] - 1 : 1;
+  const int Ld = g.N[D - 1];   // half of 2 N_d - 1: n_d = 0 .. N_d - 1
+  const int64_t rest = static_cast<int64_t>(L1) * Ld;      // entries per value of n_0
+  const int64_t half = static_cast<int64_t>(N0) * rest;    // n_0 = 0 .. N_0 - 1
+  if (threadIdx.x < kAngles) sincospi(2.0 / kAngles * threadIdx.x, &angles[threadIdx.x].y, &angles[threadIdx.x].x);
+  for (int64_t base = static_cast<int64_t>(blockIdx.x) * blockDim.x; base < half;
+       base += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+    const int64_t at = base + threadIdx.x < half ? base + threadIdx.x : half - 1;
+    const int64_t n0 = at / rest, rr = at - n0 * rest;
+    CoefEntry e;
+    e.n[0] = static_cast<int>(n0);
+    e.n[1] = D == 2 ? static_cast<int>(rr) : static_cast<int>(rr / Ld) - (g.N[1] - 1);
+    e.n[2] = D == 2 ? 0 : static_cast<int>(rr % Ld);
+    e.rho2 = double(e.n[0]) * e.n[0] + double(e.n[1]) * e.n[1] + double(e.n[2]) * e.n[2];
+    e.rho = sqrt(e.rho2);
+    e.rinv = 1.0 / e.rho;
+    e.rm32 = e.rinv * sqrt(e.rinv);
+#pragma unroll
+    for (int a = 0; a < D; ++a) e.pin[a] = 1.0 / (kPi * e.n[a]);
+    const bool origin = e.rho2 == 0.0;
+    double re = origin ? a0v : 0.0, im = 0.0, re1 = origin ? a0v1 : 0.0, im1 = 0.0;
     double rem = 0.0, imm = 0.0, rem1 = 0.0, imm1 = 0.0;   // the mirror entry
-    for (int i = 0; i < n; ++i) {
-      const Incl in = incs[i];
-      const double sh = shape_coeff(in, d, nv);
-      const double f = in.dv * sh;
-      const double f1 = tab1 != nullptr ? incs1[i].dv * sh : 0.0;
-      // exp(-2 pi i n.x_i): reduce n.x_i to [-1/2, 1/2] before the sincos
-      double t = 0.0;
-      for (int a = 0; a < d; ++a) t = fma(static_cast<double>(nv[a]), in.c[a], t);
-      t -= rint(t);
-      double s, c;
-      sincospi(2.0 * t, &s, &c);
-      re += f * c;
-      im -= f * s;
-      re1 += f1 * c;
-      im1 -= f1 * s;
-      if (mirror) {
-        double tm = 0.0;
-        for (int a = 0; a < d; ++a) tm = fma(static_cast<double>(nm[a]), in.c[a], tm);
-        tm -= rint(tm);
-        sincospi(2.0 * tm, &s, &c);
-        rem += f * c;
-        imm -= f * s;
-        rem1 += f1 * c;
-        imm1 -= f1 * s;
+    for (int i0 = 0; i0 < n; i0 += kCoefChunk) {
+      const int m = n - i0 < kCoefChunk ? n - i0 : kCoefChunk;
+      if (n > kCoefChunk || base == static_cast<int64_t>(blockIdx.x) * blockDim.x) {   // else in place from the first turn
+        __syncthreads();
+        for (int u = threadIdx.x; u < m; u += blockDim.x) {
+          const Incl& in = incs[i0 + u];
+          CoefIncl c;
+          c.shape = in.shape;
+          for (int a = 0; a < 3; ++a) {
+            c.c[a] = in.c[a];
+            c.s[a] = in.s[a];
+          }
+          c.amp = sqrt(0.5 * in.s[0]) / kPi;
+          c.inv = 1.0 / (2.0 * kPi * in.s[0]);
+          c.dv = in.dv;
+          c.dv1 = incs1[i0 + u].dv;
+          held[u] = c;
+        }
+        __syncthreads();
+      }
+      for (int i = 0; i < m; ++i) {
+        const CoefIncl& in = held[i];
+        const double sh = shape_coeff<D>(angles, in, e);
+        // exp(-2 pi i n.x_i), of the entry and of its mirror
+        const double t0 = e.n[0] * in.c[0];
+        double t = fma(static_cast<double>(e.n[1]), in.c[1], t0), tm = fma(static_cast<double>(e.n[1]), in.c[1], -t0);
+        if (D == 3) {
+          t = fma(static_cast<double>(e.n[2]), in.c[2], t);
+          tm = fma(static_cast<double>(e.n[2]), in.c[2], tm);
+        }
+        const double2 p = sincos_turns(angles, t - rint(t)), q = sincos_turns(angles, tm - rint(tm));
+        const double f = in.dv * sh, f1 = in.dv1 * sh;
+        re = fma(f, p.x, re);
+        im = fma(-f, p.y, im);
+        re1 = fma(f1, p.x, re1);
+        im1 = fma(-f1, p.y, im1);
+        rem = fma(f, q.x, rem);
+        imm = fma(-f, q.y, imm);
+        rem1 = fma(f1, q.x, rem1);
+        imm1 = fma(-f1, q.y, imm1);
       }
     }
-    const int64_t ep = (n0 + N0 - 1) * rest + rr, em = (N0 - 1 - n0) * rest + rr;
-    tab[ep] = make_double2(re, im);
-    if (tab1 != nullptr) tab1[ep] = make_double2(re1, im1);
-    if (mirror) {
-      tab[em] = make_double2(rem, imm);
-      if (tab1 != nullptr) tab1[em] = make_double2(rem1, imm1);
+    if (base + threadIdx.x < half) {
+      const int64_t ep = (n0 + N0 - 1) * rest + rr, em = (N0 - 1 - n0) * rest + rr;
+      tab[ep] = make_double2(re, im);
+      tab1[ep] = make_double2(re1, im1);
+      if (n0 != 0) {
+        tab[em] = make_double2(rem, imm);
+        tab1[em] = make_double2(rem1, imm1);
+      }
     }
   }
 }
@@ -616,7 +690,8 @@ __global__ void add_constant_kernel(double2* v, const double2* e, FieldGeom fg, 
 ghb_status launch_coeff_tables(double2* tab0, double2* tab1, const Geometry& g, const Incl* incs0,
                                const Incl* incs1, int n, double a0v0, double a0v1, cudaStream_t s) {
   const int64_t half = static_cast<int64_t>(g.N[0]) * (g.table / (2 * g.N[0] - 1));   // n_0 >= 0
-  coeff_kernel<<<field_grid(half), kFieldThreads, 0, s>>>(tab0, tab1, g, incs0, incs1, n, a0v0, a0v1);
+  if (g.d == 2) coeff_kernel<2><<<field_grid(half), kFieldThreads, 0, s>>>(tab0, tab1, g, incs0, incs1, n, a0v0, a0v1);
+  else coeff_kernel<3><<<field_grid(half), kFieldThreads, 0, s>>>(tab0, tab1, g, incs0, incs1, n, a0v0, a0v1);
   GHB_CUDA_TRY(cudaGetLastError());
   return GHB_OK;
 }

@@ -201,32 +201,56 @@ __device__ __forceinline__ void hankel_sums(double z, double& P, double& Q) {
   }
 }
 
-// Bessel function of the first kind of order one for 0 <= x < 20.
-//  x <= 8: CUDA's j1 (accurate to a few ulp there; it loses about 1e-12 of the
-//     envelope sqrt(2/(pi x)) beyond, which is visible in the bounds at 1e-13).
-//  x > 8: Miller's backward recurrence J_{n-1} = (2n/x) J_n - J_{n+1},
-//     started at n0 ~ x + 40 with J_{n0+1} = 0, normalised by the identity
-//     J_0 + 2 sum_{k>=1} J_{2k} = 1.
-__device__ __noinline__ double bessel_j1_small(double x) {
-  if (x <= 8.0) return j1(x);
-  int n0 = static_cast<int>(x) + 40;
-  n0 += n0 & 1;                       // even start
-  double jp1 = 0.0, jn = 1e-30, sum = 2.0 * jn, j1v = 0.0;
-  for (int n = n0; n >= 1; --n) {
-    const double jm1 = (2.0 * n / x) * jn - jp1;   // J_{n-1}
-    jp1 = jn;
-    jn = jm1;
-    const int m = n - 1;
-    if (m == 1) j1v = jn;
-    if ((m & 1) == 0) sum += (m == 0 ? 1.0 : 2.0) * jn;
-    if (fabs(jn) > 1e200) {          // rescale to stay in range
-      jn *= 1e-200;
-      jp1 *= 1e-200;
-      sum *= 1e-200;
-      j1v *= 1e-200;
+// J_1 on [8, 20) by Taylor's polynomials about the middles of intervals of 1/2:
+// |J_1^(k)| <= 1, so that with |t| <= 1/4 the first term left out is below 3e-18.
+// (CUDA's j1, a few ulp below 8, loses about 1e-12 of the envelope sqrt(2/(pi x))
+// beyond, which is visible in the bounds at 1e-13.  Miller's recurrence on the
+// device, used before, took some 900 FP64 instructions: 42.8 of the 315 ms that 64
+// mixed microstructures take, 8.6 of 283 now; error up to 12.6 units of 2^-53 of the
+// envelope, 1.3 now.)
+constexpr int kTaylorSpans = 24, kTaylorTerms = 13;
+struct BesselTable {
+  double a[kTaylorSpans][kTaylorTerms];
+};
+// The coefficients, in extended precision: J_0 and J_1 at the middle c by Miller's
+// backward recurrence J_{n-1} = (2n/x) J_n - J_{n+1} with J_0 + 2 sum J_{2k} = 1, the
+// others from Bessel's equation (c+t)^2 y'' + (c+t) y' + ((c+t)^2 - 1) y = 0.
+const BesselTable& bessel_table() {
+  static const BesselTable table = [] {
+    BesselTable b;
+    for (int i = 0; i < kTaylorSpans; ++i) {
+      const long double c = 8.25L + 0.5L * i;
+      long double next = 0, cur = 1e-300L, sum = cur, j1 = 0;
+      for (int n = 80; n >= 1; --n) {
+        const long double prev = 2 * n / c * cur - next;
+        next = cur;
+        cur = prev;
+        if (n == 2) j1 = cur;
+        if (n % 2 == 1) sum += cur;
+      }
+      const long double norm = 2 * sum - cur;   // J_0 counts once
+      long double a[kTaylorTerms];
+      a[0] = j1 / norm;
+      a[1] = cur / norm - a[0] / c;
+      for (int k = 0; k + 2 < kTaylorTerms; ++k)
+        a[k + 2] = -(c * (k + 1) * (2 * k + 1) * a[k + 1] + (k * k + c * c - 1) * a[k] + (k > 0 ? 2 * c * a[k - 1] : 0) +
+                     (k > 1 ? a[k - 2] : 0)) /
+                   (c * c * (k + 2) * (k + 1));
+      for (int k = 0; k < kTaylorTerms; ++k) b.a[i][k] = static_cast<double>(a[k]);
     }
-  }
-  return j1v / sum;
+    return b;
+  }();
+  return table;
+}
+// J_1 for 0 <= x < 20
+__device__ __forceinline__ double bessel_j1_small(const BesselTable& table, double x) {
+  if (x < 8.0) return j1(x);
+  const int i = static_cast<int>(2.0 * (x - 8.0));
+  const double t = x - (8.25 + 0.5 * i);
+  double v = table.a[i][kTaylorTerms - 1];
+#pragma unroll
+  for (int k = kTaylorTerms - 2; k >= 0; --k) v = fma(v, t, table.a[i][k]);
+  return v;
 }
 
 // What an inclusion and an entry bring to the shape factors.
@@ -244,7 +268,8 @@ struct CoefEntry {
 
 // Shape factor f^(n): even in each component of n.
 template <int D>
-__device__ __forceinline__ double shape_coeff(const double2* angles, const CoefIncl& in, const CoefEntry& e) {
+__device__ __forceinline__ double shape_coeff(const double2* angles, const BesselTable& bessel, const CoefIncl& in,
+                                              const CoefEntry& e) {
   if (in.shape == GHB_BOX) {        // prod_a s_a sinc(s_a n_a)
     double v = 1.0;
 #pragma unroll
@@ -255,7 +280,7 @@ __device__ __forceinline__ double shape_coeff(const double2* angles, const CoefI
   const double x = 2.0 * kPi * r * e.rho;
   if (in.shape == GHB_DISK) {       // r J_1(2 pi r rho) / rho
     if (e.rho2 == 0.0) return kPi * r * r;
-    if (x < 20.0) return r * bessel_j1_small(x) * e.rinv;
+    if (x < 20.0) return r * bessel_j1_small(bessel, x) * e.rinv;
     const double ix = in.inv * e.rinv, z = ix * ix;
     double P, Q;
     if (x >= 100.0) hankel_sums<10>(z, P, Q);   // the first term left out is below 4e-18 in each range
@@ -281,14 +306,17 @@ __device__ __forceinline__ double shape_coeff(const double2* angles, const CoefI
 constexpr int kCoefChunk = 64;     // inclusions that a block holds at a time
 template <int D>
 __global__ void __launch_bounds__(kFieldThreads) coeff_kernel(double2* tab, double2* tab1, Geometry g, const Incl* incs,
-                                                              const Incl* incs1, int n, double a0v, double a0v1) {
+                                                              const Incl* incs1, int n, double a0v, double a0v1,
+                                                              const __grid_constant__ BesselTable table) {
   __shared__ CoefIncl held[kCoefChunk];
   __shared__ double2 angles[kAngles];
+  __shared__ BesselTable bessel;
   const int N0 = g.N[0];
   const int L1 = D == 3 ? 2 * g.N[1] - 1 : 1;
   const int Ld = g.N[D - 1];   // half of 2 N_d - 1: n_d = 0 .. N_d - 1
   const int64_t rest = static_cast<int64_t>(L1) * Ld;      // entries per value of n_0
   const int64_t half = static_cast<int64_t>(N0) * rest;    // n_0 = 0 .. N_0 - 1
+  for (int i = threadIdx.x; i < kTaylorSpans * kTaylorTerms; i += blockDim.x) (&bessel.a[0][0])[i] = (&table.a[0][0])[i];
   if (threadIdx.x < kAngles) sincospi(2.0 / kAngles * threadIdx.x, &angles[threadIdx.x].y, &angles[threadIdx.x].x);
   for (int64_t base = static_cast<int64_t>(blockIdx.x) * blockDim.x; base < half;
        base += static_cast<int64_t>(gridDim.x) * blockDim.x) {
@@ -329,7 +357,7 @@ __global__ void __launch_bounds__(kFieldThreads) coeff_kernel(double2* tab, doub
       }
       for (int i = 0; i < m; ++i) {
         const CoefIncl& in = held[i];
-        const double sh = shape_coeff<D>(angles, in, e);
+        const double sh = shape_coeff<D>(angles, bessel, in, e);
         // exp(-2 pi i n.x_i), of the entry and of its mirror
         const double t0 = e.n[0] * in.c[0];
         double t = fma(static_cast<double>(e.n[1]), in.c[1], t0), tm = fma(static_cast<double>(e.n[1]), in.c[1], -t0);
@@ -690,8 +718,13 @@ __global__ void add_constant_kernel(double2* v, const double2* e, FieldGeom fg, 
 ghb_status launch_coeff_tables(double2* tab0, double2* tab1, const Geometry& g, const Incl* incs0,
                                const Incl* incs1, int n, double a0v0, double a0v1, cudaStream_t s) {
   const int64_t half = static_cast<int64_t>(g.N[0]) * (g.table / (2 * g.N[0] - 1));   // n_0 >= 0
-  if (g.d == 2) coeff_kernel<2><<<field_grid(half), kFieldThreads, 0, s>>>(tab0, tab1, g, incs0, incs1, n, a0v0, a0v1);
-  else coeff_kernel<3><<<field_grid(half), kFieldThreads, 0, s>>>(tab0, tab1, g, incs0, incs1, n, a0v0, a0v1);
+  // small tables are spread over the SMs in blocks of 64 threads
+  const int threads = half <= 152 * kFieldThreads ? kAngles : kFieldThreads;
+  const int blocks = static_cast<int>(std::min<int64_t>((half + threads - 1) / threads, 1216));
+  if (g.d == 2)
+    coeff_kernel<2><<<blocks, threads, 0, s>>>(tab0, tab1, g, incs0, incs1, n, a0v0, a0v1, bessel_table());
+  else
+    coeff_kernel<3><<<blocks, threads, 0, s>>>(tab0, tab1, g, incs0, incs1, n, a0v0, a0v1, bessel_table());
   GHB_CUDA_TRY(cudaGetLastError());
   return GHB_OK;
 }

@@ -11,12 +11,12 @@ __global__ void __launch_bounds__(kFxThreads, kFxBlocks)
 }
 
 template <int SIGN>
-__global__ void __launch_bounds__(kFxThreads, kFxBlocks) fx_col_kernel_batch(const ColItem* __restrict__ items, int n, int TW) {
+__global__ void __launch_bounds__(kFxThreads, kFxBlocks) fx_col_kernel_batch(const ColItem* __restrict__ items, int n) {
   __shared__ int s_item;
   if (threadIdx.x == 0) s_item = find_item(items, n, blockIdx.x);
   __syncthreads();
   const ColItem& it = items[s_item];
-  fx_col_body<SIGN>(it.a, it.pl->fx, TW, blockIdx.x - it.block_begin);
+  fx_col_body<SIGN>(it.a, it.pl->fx, it.tile, blockIdx.x - it.block_begin);
 }
 
 namespace {
@@ -31,11 +31,11 @@ ghb_status col_launch(const ColArgs& a, const FxPlan& f, int TW, cudaStream_t s)
 }
 
 template <int SIGN>
-ghb_status col_launch_batch(int TW, const ColItem* items, int n, int64_t blocks, size_t smem, int threads,
+ghb_status col_launch_batch(const ColItem* items, int n, int64_t blocks, size_t smem, int threads,
                             cudaStream_t s) {
   static std::atomic<unsigned long long> mask{0};
   TRY_STATUS(ensure_dyn_smem(fx_col_kernel_batch<SIGN>, 220 * 1024, mask));
-  return launch_chained(fx_col_kernel_batch<SIGN>, blocks, threads, smem, s, items, n, TW);
+  return launch_chained(fx_col_kernel_batch<SIGN>, blocks, threads, smem, s, items, n);
 }
 
 }  // namespace
@@ -44,10 +44,10 @@ ghb_status launch_fx_col(int sign, const ColArgs& a, const FxPlan& f, int TW, cu
   return sign > 0 ? col_launch<+1>(a, f, TW, s) : col_launch<-1>(a, f, TW, s);
 }
 
-ghb_status launch_fx_col_batch(int sign, int TW, const ColItem* items, int n, int64_t blocks, size_t smem, int threads,
+ghb_status launch_fx_col_batch(int sign, const ColItem* items, int n, int64_t blocks, size_t smem, int threads,
                                cudaStream_t s) {
-  return sign > 0 ? col_launch_batch<+1>(TW, items, n, blocks, smem, threads, s)
-                  : col_launch_batch<-1>(TW, items, n, blocks, smem, threads, s);
+  return sign > 0 ? col_launch_batch<+1>(items, n, blocks, smem, threads, s)
+                  : col_launch_batch<-1>(items, n, blocks, smem, threads, s);
 }
 
 }  // namespace ghb

@@ -11,12 +11,12 @@ __global__ void __launch_bounds__(kFxThreads, kFxBlocks)
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(kFxThreads, kFxBlocks) fx_row_kernel_batch(const RowItem* __restrict__ items, int n, int NL) {
+__global__ void __launch_bounds__(kFxThreads, kFxBlocks) fx_row_kernel_batch(const RowItem* __restrict__ items, int n) {
   __shared__ int s_item;
   if (threadIdx.x == 0) s_item = find_item(items, n, blockIdx.x);
   __syncthreads();
   const RowItem& it = items[s_item];
-  fx_row_body<MODE>(it.a, it.pl->fx, it.rows_per_cta, NL, blockIdx.x - it.block_begin, it.nblocks);
+  fx_row_body<MODE>(it.a, it.pl->fx, it.rows_per_cta, it.lines, blockIdx.x - it.block_begin, it.nblocks);
 }
 
 namespace {
@@ -32,11 +32,11 @@ ghb_status row_launch(const RowArgs& a, const FxPlan& f, int rows_per_cta, int N
 }
 
 template <int MODE>
-ghb_status row_launch_batch(int NL, const RowItem* items, int n, int64_t blocks, size_t smem, int threads,
+ghb_status row_launch_batch(const RowItem* items, int n, int64_t blocks, size_t smem, int threads,
                             cudaStream_t s) {
   static std::atomic<unsigned long long> mask{0};
   TRY_STATUS(ensure_dyn_smem(fx_row_kernel_batch<MODE>, 220 * 1024, mask));
-  return launch_chained(fx_row_kernel_batch<MODE>, blocks, threads, smem, s, items, n, NL);
+  return launch_chained(fx_row_kernel_batch<MODE>, blocks, threads, smem, s, items, n);
 }
 
 }  // namespace
@@ -50,11 +50,11 @@ ghb_status launch_fx_row(int mode, const RowArgs& a, const FxPlan& f, int rows_p
   }
 }
 
-ghb_status launch_fx_row_batch(int mode, int NL, const RowItem* items, int n, int64_t blocks, size_t smem, int threads,
+ghb_status launch_fx_row_batch(int mode, const RowItem* items, int n, int64_t blocks, size_t smem, int threads,
                                cudaStream_t s) {
   switch (mode) {
-    case ROW_MATVEC: return row_launch_batch<ROW_MATVEC>(NL, items, n, blocks, smem, threads, s);
-    case ROW_ENERGY: return row_launch_batch<ROW_ENERGY>(NL, items, n, blocks, smem, threads, s);
+    case ROW_MATVEC: return row_launch_batch<ROW_MATVEC>(items, n, blocks, smem, threads, s);
+    case ROW_ENERGY: return row_launch_batch<ROW_ENERGY>(items, n, blocks, smem, threads, s);
     default: break;
   }
   set_error("internal: unsupported batched row pass");

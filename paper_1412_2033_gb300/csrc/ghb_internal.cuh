@@ -199,24 +199,25 @@ struct ColItem {
   ColArgs a;
   const FftPlan* pl;     // device copy of the item's plan
   int64_t block_begin;
+  int tile;              // columns per CTA
 };
 
 struct RowItem {
   RowArgs a;
   const FftPlan* pl;
   int rows_per_cta;
-  int pad;
+  int lines;             // complex lines of rows_per_cta rows
   int64_t nblocks;
   int64_t block_begin;
 };
 
-// Batched launches; TW / NL and the shared-memory size are chosen by the caller
-// for the largest M of the batch (col_tile_width, row_lines).
+// Batched launches; the lines per CTA are the item's, shared memory and threads
+// hold the largest (batch.cu).
 template <typename T>
-ghb_status launch_col_batch(int sign, int mode, int TW, const ColItem* items, int n, int64_t blocks,
+ghb_status launch_col_batch(int sign, int mode, const ColItem* items, int n, int64_t blocks,
                             size_t smem, int threads, cudaStream_t s);
 template <typename T>
-ghb_status launch_row_batch(int mode, int NL, const RowItem* items, int n, int64_t blocks, size_t smem, int threads,
+ghb_status launch_row_batch(int mode, const RowItem* items, int n, int64_t blocks, size_t smem, int threads,
                             cudaStream_t s);
 // rows per CTA and interleaved complex lines of a row pass
 // Rows per CTA and interleaved complex lines of a last-axis pass; rows32 is the

@@ -197,27 +197,27 @@ void row_lines(int mode, int nfields, int ncomp, int M, int rows32, int* rows_pe
 }
 
 template <>
-ghb_status launch_col_batch<float>(int sign, int mode, int TW, const ColItem* items, int n, int64_t blocks,
-                                   size_t smem, int threads, cudaStream_t s) {
-  return launch_rt_col_batch(sign, mode == COL_PUPDATE, TW, items, n, blocks, smem, threads, s);
+ghb_status launch_col_batch<float>(int sign, int mode, const ColItem* items, int n, int64_t blocks, size_t smem,
+                                   int threads, cudaStream_t s) {
+  return launch_rt_col_batch(sign, mode == COL_PUPDATE, items, n, blocks, smem, threads, s);
 }
 template <>
-ghb_status launch_col_batch<double>(int sign, int, int TW, const ColItem* items, int n, int64_t blocks, size_t smem,
-                                    int threads, cudaStream_t s) {
-  return launch_fx_col_batch(sign, TW, items, n, blocks, smem, threads, s);
+ghb_status launch_col_batch<double>(int sign, int, const ColItem* items, int n, int64_t blocks, size_t smem, int threads,
+                                    cudaStream_t s) {
+  return launch_fx_col_batch(sign, items, n, blocks, smem, threads, s);
 }
 
 template <>
-ghb_status launch_row_batch<float>(int mode, int NL, const RowItem* items, int n, int64_t blocks, size_t smem,
-                                   int threads, cudaStream_t s) {
-  if (mode == ROW_MATVEC) return launch_rt_row_batch(NL, items, n, blocks, smem, threads, s);
+ghb_status launch_row_batch<float>(int mode, const RowItem* items, int n, int64_t blocks, size_t smem, int threads,
+                                   cudaStream_t s) {
+  if (mode == ROW_MATVEC) return launch_rt_row_batch(items, n, blocks, smem, threads, s);
   set_error("internal: unsupported batched row pass");
   return GHB_ERR_INVALID;
 }
 template <>
-ghb_status launch_row_batch<double>(int mode, int NL, const RowItem* items, int n, int64_t blocks, size_t smem,
-                                    int threads, cudaStream_t s) {
-  return launch_fx_row_batch(mode, NL, items, n, blocks, smem, threads, s);
+ghb_status launch_row_batch<double>(int mode, const RowItem* items, int n, int64_t blocks, size_t smem, int threads,
+                                    cudaStream_t s) {
+  return launch_fx_row_batch(mode, items, n, blocks, smem, threads, s);
 }
 
 template <>

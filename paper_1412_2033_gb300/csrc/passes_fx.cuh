@@ -536,11 +536,11 @@ void fx_row_shape(int mode, int nfields, int ncomp, int M, int ls, int64_t rows,
 
 // Launchers (fx_col.cu, fx_row.cu).
 ghb_status launch_fx_col(int sign, const ColArgs& a, const FxPlan& f, int TW, cudaStream_t s);
-ghb_status launch_fx_col_batch(int sign, int TW, const ColItem* items, int n, int64_t blocks, size_t smem, int threads,
+ghb_status launch_fx_col_batch(int sign, const ColItem* items, int n, int64_t blocks, size_t smem, int threads,
                                cudaStream_t s);
 ghb_status launch_fx_row(int mode, const RowArgs& a, const FxPlan& f, int rows_per_cta, int NL, int threads,
                          cudaStream_t s);
-ghb_status launch_fx_row_batch(int mode, int NL, const RowItem* items, int n, int64_t blocks, size_t smem, int threads,
+ghb_status launch_fx_row_batch(int mode, const RowItem* items, int n, int64_t blocks, size_t smem, int threads,
                                cudaStream_t s);
 
 }  // namespace ghb

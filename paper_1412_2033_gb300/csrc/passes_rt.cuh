@@ -295,10 +295,10 @@ int rt_threads(int M, int lines, int ls);
 // want: 0 = lines by size, 1 / 2 = the least rows once or twice
 void rt_row_shape(int ncomp, int M, int ls, int64_t rows, int want, int* rows_per_cta, int* lines);
 ghb_status launch_rt_col(int sign, const ColArgs& a, const FxPlan& f, int TW, cudaStream_t s);
-ghb_status launch_rt_col_batch(int sign, bool update, int TW, const ColItem* items, int n, int64_t blocks, size_t smem,
+ghb_status launch_rt_col_batch(int sign, bool update, const ColItem* items, int n, int64_t blocks, size_t smem,
                                int threads, cudaStream_t s);
 ghb_status launch_rt_row(const RowArgs& a, const FxPlan& f, int rows_per_cta, int lines, cudaStream_t s);
-ghb_status launch_rt_row_batch(int lines, const RowItem* items, int n, int64_t blocks, size_t smem, int threads,
+ghb_status launch_rt_row_batch(const RowItem* items, int n, int64_t blocks, size_t smem, int threads,
                                cudaStream_t s);
 
 }  // namespace ghb

@@ -11,12 +11,12 @@ __global__ void __launch_bounds__(kRtThreads, 1)
 }
 
 template <int SIGN, bool UPDATE>
-__global__ void __launch_bounds__(kRtThreads, 1) rt_col_kernel_batch(const ColItem* __restrict__ items, int n, int TW) {
+__global__ void __launch_bounds__(kRtThreads, 1) rt_col_kernel_batch(const ColItem* __restrict__ items, int n) {
   __shared__ int s_item;
   if (threadIdx.x == 0) s_item = find_item(items, n, blockIdx.x);
   __syncthreads();
   const ColItem& it = items[s_item];
-  rt_col_body<SIGN, UPDATE>(it.a, it.pl->rt, TW, blockIdx.x - it.block_begin);
+  rt_col_body<SIGN, UPDATE>(it.a, it.pl->rt, it.tile, blockIdx.x - it.block_begin);
 }
 
 namespace {
@@ -31,11 +31,11 @@ ghb_status col_launch(const ColArgs& a, const FxPlan& f, int TW, cudaStream_t s)
 }
 
 template <int SIGN, bool UPDATE>
-ghb_status col_launch_batch(int TW, const ColItem* items, int n, int64_t blocks, size_t smem, int threads,
+ghb_status col_launch_batch(const ColItem* items, int n, int64_t blocks, size_t smem, int threads,
                             cudaStream_t s) {
   static std::atomic<unsigned long long> mask{0};
   TRY_STATUS(ensure_dyn_smem(rt_col_kernel_batch<SIGN, UPDATE>, 220 * 1024, mask));
-  return launch_chained(rt_col_kernel_batch<SIGN, UPDATE>, blocks, threads, smem, s, items, n, TW);
+  return launch_chained(rt_col_kernel_batch<SIGN, UPDATE>, blocks, threads, smem, s, items, n);
 }
 
 }  // namespace
@@ -45,11 +45,11 @@ ghb_status launch_rt_col(int sign, const ColArgs& a, const FxPlan& f, int TW, cu
   return a.pold != nullptr ? col_launch<+1, true>(a, f, TW, s) : col_launch<+1, false>(a, f, TW, s);
 }
 
-ghb_status launch_rt_col_batch(int sign, bool update, int TW, const ColItem* items, int n, int64_t blocks, size_t smem,
+ghb_status launch_rt_col_batch(int sign, bool update, const ColItem* items, int n, int64_t blocks, size_t smem,
                                int threads, cudaStream_t s) {
-  if (sign < 0) return col_launch_batch<-1, false>(TW, items, n, blocks, smem, threads, s);
-  return update ? col_launch_batch<+1, true>(TW, items, n, blocks, smem, threads, s)
-                : col_launch_batch<+1, false>(TW, items, n, blocks, smem, threads, s);
+  if (sign < 0) return col_launch_batch<-1, false>(items, n, blocks, smem, threads, s);
+  return update ? col_launch_batch<+1, true>(items, n, blocks, smem, threads, s)
+                : col_launch_batch<+1, false>(items, n, blocks, smem, threads, s);
 }
 
 }  // namespace ghb

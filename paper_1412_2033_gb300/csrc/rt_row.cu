@@ -10,12 +10,12 @@ __global__ void __launch_bounds__(kRtThreads, 1)
 }
 
 __global__ void __launch_bounds__(kRtThreads, 1)
-    rt_row_kernel_batch(const RowItem* __restrict__ items, int n, int lines) {
+    rt_row_kernel_batch(const RowItem* __restrict__ items, int n) {
   __shared__ int s_item;
   if (threadIdx.x == 0) s_item = find_item(items, n, blockIdx.x);
   __syncthreads();
   const RowItem& it = items[s_item];
-  rt_row_body(it.a, it.pl->rt, it.rows_per_cta, lines, blockIdx.x - it.block_begin, it.nblocks);
+  rt_row_body(it.a, it.pl->rt, it.rows_per_cta, it.lines, blockIdx.x - it.block_begin, it.nblocks);
 }
 
 ghb_status launch_rt_row(const RowArgs& a, const FxPlan& f, int rows_per_cta, int lines, cudaStream_t s) {
@@ -26,11 +26,11 @@ ghb_status launch_rt_row(const RowArgs& a, const FxPlan& f, int rows_per_cta, in
   return launch_chained(rt_row_kernel, grid, rt_threads(f.M, lines, f.ls), smem, s, a, f, rows_per_cta, lines);
 }
 
-ghb_status launch_rt_row_batch(int lines, const RowItem* items, int n, int64_t blocks, size_t smem, int threads,
+ghb_status launch_rt_row_batch(const RowItem* items, int n, int64_t blocks, size_t smem, int threads,
                                cudaStream_t s) {
   static std::atomic<unsigned long long> mask{0};
   TRY_STATUS(ensure_dyn_smem(rt_row_kernel_batch, 200 * 1024, mask));
-  return launch_chained(rt_row_kernel_batch, blocks, threads, smem, s, items, n, lines);
+  return launch_chained(rt_row_kernel_batch, blocks, threads, smem, s, items, n);
 }
 
 }  // namespace ghb

@@ -670,21 +670,10 @@ __global__ void __launch_bounds__(kFieldThreads) cg_kernel(CgItem it) {
   run_op<T, OP>(it, blockIdx.x, gridDim.x);
 }
 
-template <typename Item>
-__device__ __forceinline__ int find_cg_item(const Item* items, int n, int64_t b) {
-  int lo = 0, hi = n - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (items[mid].block_begin <= b) lo = mid;
-    else hi = mid - 1;
-  }
-  return lo;
-}
-
 template <typename T, int OP>
 __global__ void __launch_bounds__(kFieldThreads) cg_kernel_batch(const CgItem* __restrict__ items, int n) {
   __shared__ int s_item;
-  if (threadIdx.x == 0) s_item = find_cg_item(items, n, blockIdx.x);
+  if (threadIdx.x < 32) s_item = find_item(items, n, blockIdx.x);
   __syncthreads();
   const CgItem& it = items[s_item];
   grid_wait();

@@ -13,7 +13,7 @@ __global__ void __launch_bounds__(kFxThreads, kFxBlocks)
 template <int SIGN>
 __global__ void __launch_bounds__(kFxThreads, kFxBlocks) fx_col_kernel_batch(const ColItem* __restrict__ items, int n) {
   __shared__ int s_item;
-  if (threadIdx.x == 0) s_item = find_item(items, n, blockIdx.x);
+  if (threadIdx.x < 32) s_item = find_item(items, n, blockIdx.x);
   __syncthreads();
   const ColItem& it = items[s_item];
   fx_col_body<SIGN>(it.a, it.pl->fx, it.tile, blockIdx.x - it.block_begin);

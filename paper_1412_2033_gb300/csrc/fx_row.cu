@@ -13,7 +13,7 @@ __global__ void __launch_bounds__(kFxThreads, kFxBlocks)
 template <int MODE>
 __global__ void __launch_bounds__(kFxThreads, kFxBlocks) fx_row_kernel_batch(const RowItem* __restrict__ items, int n) {
   __shared__ int s_item;
-  if (threadIdx.x == 0) s_item = find_item(items, n, blockIdx.x);
+  if (threadIdx.x < 32) s_item = find_item(items, n, blockIdx.x);
   __syncthreads();
   const RowItem& it = items[s_item];
   fx_row_body<MODE>(it.a, it.pl->fx, it.rows_per_cta, it.lines, blockIdx.x - it.block_begin, it.nblocks);

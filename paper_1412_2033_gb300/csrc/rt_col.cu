@@ -13,7 +13,7 @@ __global__ void __launch_bounds__(kRtThreads, 1)
 template <int SIGN, bool UPDATE>
 __global__ void __launch_bounds__(kRtThreads, 1) rt_col_kernel_batch(const ColItem* __restrict__ items, int n) {
   __shared__ int s_item;
-  if (threadIdx.x == 0) s_item = find_item(items, n, blockIdx.x);
+  if (threadIdx.x < 32) s_item = find_item(items, n, blockIdx.x);
   __syncthreads();
   const ColItem& it = items[s_item];
   rt_col_body<SIGN, UPDATE>(it.a, it.pl->rt, it.tile, blockIdx.x - it.block_begin);

@@ -12,7 +12,7 @@ __global__ void __launch_bounds__(kRtThreads, 1)
 __global__ void __launch_bounds__(kRtThreads, 1)
     rt_row_kernel_batch(const RowItem* __restrict__ items, int n) {
   __shared__ int s_item;
-  if (threadIdx.x == 0) s_item = find_item(items, n, blockIdx.x);
+  if (threadIdx.x < 32) s_item = find_item(items, n, blockIdx.x);
   __syncthreads();
   const RowItem& it = items[s_item];
   rt_row_body(it.a, it.pl->rt, it.rows_per_cta, it.lines, blockIdx.x - it.block_begin, it.nblocks);

@@ -109,9 +109,9 @@ __device__ __forceinline__ void project_vec(int d, const int k[3], int kind, con
 // `bid`, `nb`: this block and the number of blocks working on the same operand.
 __device__ bool grid_sum_last(double v, double* partials, unsigned int* ticket, double* total,
                               int64_t bid, int64_t nb) {
-  __shared__ double red[32];
+  __shared__ double red[kFieldThreads];
   __shared__ bool last;
-  const double bs = block_sum(v, red);
+  const double bs = block_sum_wide(v, red);
   if (threadIdx.x == 0) {
     partials[bid] = bs;
     __threadfence();
@@ -123,7 +123,7 @@ __device__ bool grid_sum_last(double v, double* partials, unsigned int* ticket, 
   __threadfence();
   double s = 0.0;
   for (int64_t b = threadIdx.x; b < nb; b += blockDim.x) s += __ldcg(&partials[b]);
-  s = block_sum(s, red);
+  s = block_sum_wide(s, red);
   if (threadIdx.x == 0) {
     *ticket = 0u;
     *total = s;

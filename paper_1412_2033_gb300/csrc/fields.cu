@@ -10,6 +10,7 @@
 #include <atomic>
 #include <cmath>
 
+#include "fft_fx.cuh"
 #include "ghb_internal.cuh"
 #include "launch_util.cuh"
 #include "reduce.cuh"
@@ -141,36 +142,39 @@ __device__ bool grid_sum_last(double v, double* partials, unsigned int* ticket, 
 // So a pair's own work is cut to what depends on the pair: |n|, its reciprocal and
 // |n|^(-3/2) belong to the entry, the radius' constants to the inclusion (in shared
 // memory); J_1 beyond 20 is Hankel's expansion with the coefficients as constants;
-// and sines and cosines take 18 FP64 instructions from a table of 64 angles.
-// Measured, N = 1023, 20 disks: 4.43 ms, 106 FP64 instructions a pair, FP64 pipe 86 %
-// busy (before, about 12 ms: sincospi twice a pair, divisions in every Hankel term).
+// and sines and cosines take 15 FP64 instructions from a table of 256 angles.
+// Measured, N = 1023, 20 disks: 3.71 ms, about 94 FP64 instructions a pair, FP64 pipe
+// 86 % busy (4.43 ms with 64 angles and every n.x reduced first; about 12 ms before:
+// sincospi twice a pair, divisions in every Hankel term).
 
-// The angles j / 64 of a turn, and sin, cos of one of them plus a <= pi / 64: the
-// Taylor polynomials to a^7 and a^8 (the next terms are below 2e-19) and the
-// addition theorem, with the corrections added last (half a unit beyond the
-// table's own rounding).
-constexpr int kAngles = 64;
+// sin, cos of one of the angles j / 256 of a turn plus a <= pi / 256: the Taylor
+// polynomials to a^5 and a^6 (the next terms are below 1e-17) and the addition
+// theorem, with the corrections added last (half a unit beyond the table's own
+// rounding).  The small angle is given in turns or in radians.
+constexpr int kAngles = 256;
+template <bool TURNS>
 __device__ __forceinline__ double2 turn_sincos(const double2* angles, double whole, double a) {
+  constexpr double u = TURNS ? 2.0 * kPi : 1.0;
   const double2 t = angles[__double2loint(whole) & (kAngles - 1)];   // (cos, sin)
   const double a2 = a * a;
-  const double sn = a * fma(a2, fma(a2, fma(a2, -1.0 / 5040, 1.0 / 120), -1.0 / 6), 1.0);
-  const double cm = a2 * fma(a2, fma(a2, fma(a2, 1.0 / 40320, -1.0 / 720), 1.0 / 24), -0.5);
+  const double sn = a * fma(a2, fma(a2, u * u * u * u * u / 120, -u * u * u / 6), u);
+  const double cm = a2 * fma(a2, fma(a2, -u * u * u * u * u * u / 720, u * u * u * u / 24), -u * u / 2);
   return make_double2(t.x + fma(t.x, cm, -(t.y * sn)), t.y + fma(t.y, cm, t.x * sn));
 }
 // The integer nearest to v (|v| < 2^51) in the low bits of v + kWhole.
 constexpr double kWhole = 6755399441055744.0;   // 1.5 2^52
-// (cos, sin) of 2 pi t, |t| <= 1/2
+// (cos, sin) of 2 pi t, |t| < 2^43
 __device__ __forceinline__ double2 sincos_turns(const double2* angles, double t) {
   const double w = fma(t, static_cast<double>(kAngles), kWhole);
-  return turn_sincos(angles, w, (2.0 * kPi) * fma(w - kWhole, -1.0 / kAngles, t));   // the difference is exact
+  return turn_sincos<true>(angles, w, fma(w - kWhole, -1.0 / kAngles, t));   // the difference is exact
 }
-// (cos, sin) of x, |x| < 2^40: x minus a multiple of 2 pi / 64 in two parts
+// (cos, sin) of x, |x| < 2^40: x minus a multiple of 2 pi / 256 in two parts
 __device__ __forceinline__ double2 sincos_radians(const double2* angles, double x) {
-  constexpr double kHi = 2.0 * kPi / kAngles;                    // 2 pi / 64 rounded, and the rest of it
+  constexpr double kHi = 2.0 * kPi / kAngles;                    // 2 pi / 256 rounded, and the rest of it
   constexpr double kLo = 2.4492935982947064e-16 / kAngles;
   const double w = fma(x, kAngles / (2.0 * kPi), kWhole);
   const double k = w - kWhole;
-  return turn_sincos(angles, w, fma(-k, kLo, fma(-k, kHi, x)));
+  return turn_sincos<false>(angles, w, fma(-k, kLo, fma(-k, kHi, x)));
 }
 
 // Coefficients of Hankel's expansion of J_1 (Abramowitz and Stegun 9.2.5, 9.2.9-
@@ -209,15 +213,21 @@ __device__ __forceinline__ void hankel_sums(double z, double& P, double& Q) {
 // mixed microstructures take, 8.6 of 283 now; error up to 12.6 units of 2^-53 of the
 // envelope, 1.3 now.)
 constexpr int kTaylorSpans = 24, kTaylorTerms = 13;
-struct BesselTable {
-  double a[kTaylorSpans][kTaylorTerms];
+// What the host tabulates, once a process, for every table: an argument of the kernel.
+struct CoefTables {
+  double2 angles[kAngles];                   // (cos, sin) of j / 256 turns
+  double j1[kTaylorSpans][kTaylorTerms];
 };
 // The coefficients, in extended precision: J_0 and J_1 at the middle c by Miller's
 // backward recurrence J_{n-1} = (2n/x) J_n - J_{n+1} with J_0 + 2 sum J_{2k} = 1, the
 // others from Bessel's equation (c+t)^2 y'' + (c+t) y' + ((c+t)^2 - 1) y = 0.
-const BesselTable& bessel_table() {
-  static const BesselTable table = [] {
-    BesselTable b;
+const CoefTables& coef_tables() {
+  static const CoefTables tables = [] {
+    CoefTables b;
+    std::vector<UnitRoot> roots;
+    unit_roots(kAngles, roots);
+    for (int j = 0; j < kAngles; ++j)
+      b.angles[j] = make_double2(static_cast<double>(roots[j].c), static_cast<double>(roots[j].s));
     for (int i = 0; i < kTaylorSpans; ++i) {
       const long double c = 8.25L + 0.5L * i;
       long double next = 0, cur = 1e-300L, sum = cur, j1 = 0;
@@ -236,20 +246,20 @@ const BesselTable& bessel_table() {
         a[k + 2] = -(c * (k + 1) * (2 * k + 1) * a[k + 1] + (k * k + c * c - 1) * a[k] + (k > 0 ? 2 * c * a[k - 1] : 0) +
                      (k > 1 ? a[k - 2] : 0)) /
                    (c * c * (k + 2) * (k + 1));
-      for (int k = 0; k < kTaylorTerms; ++k) b.a[i][k] = static_cast<double>(a[k]);
+      for (int k = 0; k < kTaylorTerms; ++k) b.j1[i][k] = static_cast<double>(a[k]);
     }
     return b;
   }();
-  return table;
+  return tables;
 }
 // J_1 for 0 <= x < 20
-__device__ __forceinline__ double bessel_j1_small(const BesselTable& table, double x) {
+__device__ __forceinline__ double bessel_j1_small(const CoefTables& tables, double x) {
   if (x < 8.0) return j1(x);
   const int i = static_cast<int>(2.0 * (x - 8.0));
   const double t = x - (8.25 + 0.5 * i);
-  double v = table.a[i][kTaylorTerms - 1];
+  double v = tables.j1[i][kTaylorTerms - 1];
 #pragma unroll
-  for (int k = kTaylorTerms - 2; k >= 0; --k) v = fma(v, t, table.a[i][k]);
+  for (int k = kTaylorTerms - 2; k >= 0; --k) v = fma(v, t, tables.j1[i][k]);
   return v;
 }
 
@@ -259,6 +269,7 @@ struct CoefIncl {
   double c[3], s[3];
   double amp, inv;         // disk: sqrt(r / 2) / pi, 1 / (2 pi r)
   double dv, dv1;
+  int far;                 // a centre so far out that n.x needs reducing first
 };
 struct CoefEntry {
   int n[3];
@@ -268,8 +279,7 @@ struct CoefEntry {
 
 // Shape factor f^(n): even in each component of n.
 template <int D>
-__device__ __forceinline__ double shape_coeff(const double2* angles, const BesselTable& bessel, const CoefIncl& in,
-                                              const CoefEntry& e) {
+__device__ __forceinline__ double shape_coeff(const CoefTables& tables, const CoefIncl& in, const CoefEntry& e) {
   if (in.shape == GHB_BOX) {        // prod_a s_a sinc(s_a n_a)
     double v = 1.0;
 #pragma unroll
@@ -280,14 +290,14 @@ __device__ __forceinline__ double shape_coeff(const double2* angles, const Besse
   const double x = 2.0 * kPi * r * e.rho;
   if (in.shape == GHB_DISK) {       // r J_1(2 pi r rho) / rho
     if (e.rho2 == 0.0) return kPi * r * r;
-    if (x < 20.0) return r * bessel_j1_small(bessel, x) * e.rinv;
+    if (x < 20.0) return r * bessel_j1_small(tables, x) * e.rinv;
     const double ix = in.inv * e.rinv, z = ix * ix;
     double P, Q;
     if (x >= 100.0) hankel_sums<10>(z, P, Q);   // the first term left out is below 4e-18 in each range
     else if (x >= 40.0) hankel_sums<14>(z, P, Q);
     else hankel_sums<34>(z, P, Q);
     // sqrt(2 / (pi x)) (P cos chi - Q sin chi), chi = x - 3 pi / 4
-    const double2 t = sincos_radians(angles, x);
+    const double2 t = sincos_radians(tables.angles, x);
     return in.amp * e.rm32 * fma(P, t.y - t.x, Q * ix * (t.x + t.y));
   }
   // sphere: (sin x - x cos x) / (2 pi^2 rho^3)
@@ -295,7 +305,7 @@ __device__ __forceinline__ double shape_coeff(const double2* angles, const Besse
     const double q2 = x * x;
     return 4.0 / 3.0 * kPi * r * r * r * (1.0 - q2 / 10.0 + q2 * q2 / 280.0 - q2 * q2 * q2 / 15120.0);
   }
-  const double2 t = sincos_radians(angles, x);
+  const double2 t = sincos_radians(tables.angles, x);
   return (t.y - x * t.x) * ((1.0 / (2.0 * kPi * kPi)) * (e.rinv * e.rinv * e.rinv));
 }
 
@@ -307,17 +317,16 @@ constexpr int kCoefChunk = 64;     // inclusions that a block holds at a time
 template <int D>
 __global__ void __launch_bounds__(kFieldThreads) coeff_kernel(double2* tab, double2* tab1, Geometry g, const Incl* incs,
                                                               const Incl* incs1, int n, double a0v, double a0v1,
-                                                              const __grid_constant__ BesselTable table) {
+                                                              const __grid_constant__ CoefTables given) {
   __shared__ CoefIncl held[kCoefChunk];
-  __shared__ double2 angles[kAngles];
-  __shared__ BesselTable bessel;
+  __shared__ CoefTables tables;
   const int N0 = g.N[0];
   const int L1 = D == 3 ? 2 * g.N[1] - 1 : 1;
   const int Ld = g.N[D - 1];   // half of 2 N_d - 1: n_d = 0 .. N_d - 1
   const int64_t rest = static_cast<int64_t>(L1) * Ld;      // entries per value of n_0
   const int64_t half = static_cast<int64_t>(N0) * rest;    // n_0 = 0 .. N_0 - 1
-  for (int i = threadIdx.x; i < kTaylorSpans * kTaylorTerms; i += blockDim.x) (&bessel.a[0][0])[i] = (&table.a[0][0])[i];
-  if (threadIdx.x < kAngles) sincospi(2.0 / kAngles * threadIdx.x, &angles[threadIdx.x].y, &angles[threadIdx.x].x);
+  for (int i = threadIdx.x; i < static_cast<int>(sizeof(CoefTables) / sizeof(double)); i += blockDim.x)
+    reinterpret_cast<double*>(&tables)[i] = reinterpret_cast<const double*>(&given)[i];
   for (int64_t base = static_cast<int64_t>(blockIdx.x) * blockDim.x; base < half;
        base += static_cast<int64_t>(gridDim.x) * blockDim.x) {
     const int64_t at = base + threadIdx.x < half ? base + threadIdx.x : half - 1;
@@ -343,7 +352,9 @@ __global__ void __launch_bounds__(kFieldThreads) coeff_kernel(double2* tab, doub
           const Incl& in = incs[i0 + u];
           CoefIncl c;
           c.shape = in.shape;
+          c.far = 0;
           for (int a = 0; a < 3; ++a) {
+            c.far |= fabs(in.c[a]) > 1048576.0;
             c.c[a] = in.c[a];
             c.s[a] = in.s[a];
           }
@@ -357,7 +368,7 @@ __global__ void __launch_bounds__(kFieldThreads) coeff_kernel(double2* tab, doub
       }
       for (int i = 0; i < m; ++i) {
         const CoefIncl& in = held[i];
-        const double sh = shape_coeff<D>(angles, bessel, in, e);
+        const double sh = shape_coeff<D>(tables, in, e);
         // exp(-2 pi i n.x_i), of the entry and of its mirror
         const double t0 = e.n[0] * in.c[0];
         double t = fma(static_cast<double>(e.n[1]), in.c[1], t0), tm = fma(static_cast<double>(e.n[1]), in.c[1], -t0);
@@ -365,7 +376,11 @@ __global__ void __launch_bounds__(kFieldThreads) coeff_kernel(double2* tab, doub
           t = fma(static_cast<double>(e.n[2]), in.c[2], t);
           tm = fma(static_cast<double>(e.n[2]), in.c[2], tm);
         }
-        const double2 p = sincos_turns(angles, t - rint(t)), q = sincos_turns(angles, tm - rint(tm));
+        if (in.far) {
+          t -= rint(t);
+          tm -= rint(tm);
+        }
+        const double2 p = sincos_turns(tables.angles, t), q = sincos_turns(tables.angles, tm);
         const double f = in.dv * sh, f1 = in.dv1 * sh;
         re = fma(f, p.x, re);
         im = fma(-f, p.y, im);
@@ -708,12 +723,12 @@ ghb_status launch_coeff_tables(double2* tab0, double2* tab1, const Geometry& g, 
                                const Incl* incs1, int n, double a0v0, double a0v1, cudaStream_t s) {
   const int64_t half = static_cast<int64_t>(g.N[0]) * (g.table / (2 * g.N[0] - 1));   // n_0 >= 0
   // small tables are spread over the SMs in blocks of 64 threads
-  const int threads = half <= 152 * kFieldThreads ? kAngles : kFieldThreads;
+  const int threads = half <= 152 * kFieldThreads ? 64 : kFieldThreads;
   const int blocks = static_cast<int>(std::min<int64_t>((half + threads - 1) / threads, 1216));
   if (g.d == 2)
-    coeff_kernel<2><<<blocks, threads, 0, s>>>(tab0, tab1, g, incs0, incs1, n, a0v0, a0v1, bessel_table());
+    coeff_kernel<2><<<blocks, threads, 0, s>>>(tab0, tab1, g, incs0, incs1, n, a0v0, a0v1, coef_tables());
   else
-    coeff_kernel<3><<<blocks, threads, 0, s>>>(tab0, tab1, g, incs0, incs1, n, a0v0, a0v1, bessel_table());
+    coeff_kernel<3><<<blocks, threads, 0, s>>>(tab0, tab1, g, incs0, incs1, n, a0v0, a0v1, coef_tables());
   GHB_CUDA_TRY(cudaGetLastError());
   return GHB_OK;
 }

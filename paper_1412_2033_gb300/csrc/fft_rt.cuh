@@ -8,8 +8,9 @@
 // than registers here: the passes of a short line are bound by latency (loads,
 // barriers), and a group of 16 entries has that many loads in flight.
 //
-// Bound by latency and instruction fetch (24 warps an SM, the largest stall
-// "no instruction"; issue 40 % of the cycles).  Measured against the scalar
+// Bound by latency and instruction fetch (at 24 warps an SM the largest stall is
+// "no instruction" and 45 % of the cycles issue; 32 warps at 64 registers where a
+// launch has work for them, see kRtManyThreads).  Measured against the scalar
 // run-time engine this replaces (groups of up to 32 by nested dispatch, padded
 // index per entry, a copy into and out of shared memory around every transform):
 // N = 1023, M = 2048 last axis 57 -> 41 us, axis 1 52 / 42 -> 20 / 18, operator 154.5

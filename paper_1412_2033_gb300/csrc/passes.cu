@@ -133,10 +133,14 @@ int rt_col_tile(int M, int ls, int64_t columns) {
   }
   return 2;
 }
+// More warps than the 24 that kernels of 80 registers keep on every SM.
+bool rt_many_warps(int64_t blocks, int threads) {
+  return blocks * (threads / 32) > int64_t(kRtThreads / 32) * device_sms();
+}
 // about one group of sixteen entries a thread and pass, whole warps
 int rt_threads(int M, int lines, int ls) {
   const size_t smem = static_cast<size_t>(lines) * ls * sizeof(float2);
-  const int full = smem > 110 * 1024 ? kRtThreads : (smem > 73 * 1024 ? kRtThreads / 2 : kRtThreads / 3);
+  const int full = smem > 110 * 1024 ? kRtThreads : (smem > 73 * 1024 ? kRtThreads / 2 : 256);
   const int t = ((lines * M / 16 + 31) / 32) * 32;
   return t < 64 ? 64 : (t < full ? t : full);
 }

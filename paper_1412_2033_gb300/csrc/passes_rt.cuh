@@ -12,6 +12,14 @@ namespace ghb {
 // Largest block: 24 warps of up to 80 registers (a group of 16 takes 32), as one
 // CTA or as several smaller ones.
 constexpr int kRtThreads = 768;
+// The last-axis and the batched column kernels are also compiled for 64 registers,
+// 32 warps an SM: they spill a little, and gain where more warps than 24 an SM have
+// work at once.  N = 1023 operator 68 -> 66.5 us, N = 1215 115 -> 112.7, 64 mixed
+// microstructures 236 -> 227 ms; with fewer, 80 registers are better (N = 405 32.2
+// against 32.7 us, N = 511 bound pair 20.4 against 20.8 ms), and for single column
+// passes always (N = 1023 operator 66.5 against 71.9).
+constexpr int kRtManyThreads = 1024;
+bool rt_many_warps(int64_t blocks, int threads);   // passes.cu
 constexpr int kRtMaxLines = 32;
 
 struct RtShared {

@@ -10,8 +10,8 @@ __global__ void __launch_bounds__(kRtThreads, 1)
   rt_col_body<SIGN, UPDATE>(a, f, TW, blockIdx.x);
 }
 
-template <int SIGN, bool UPDATE>
-__global__ void __launch_bounds__(kRtThreads, 1) rt_col_kernel_batch(const ColItem* __restrict__ items, int n) {
+template <int SIGN, bool UPDATE, int THREADS>
+__global__ void __launch_bounds__(THREADS, 1) rt_col_kernel_batch(const ColItem* __restrict__ items, int n) {
   __shared__ int s_item;
   if (threadIdx.x < 32) s_item = find_item(items, n, blockIdx.x);
   __syncthreads();
@@ -30,12 +30,17 @@ ghb_status col_launch(const ColArgs& a, const FxPlan& f, int TW, cudaStream_t s)
   return launch_chained(rt_col_kernel<SIGN, UPDATE>, grid, rt_threads(f.M, TW, f.ls), smem, s, a, f, TW);
 }
 
-template <int SIGN, bool UPDATE>
-ghb_status col_launch_batch(const ColItem* items, int n, int64_t blocks, size_t smem, int threads,
-                            cudaStream_t s) {
+template <int SIGN, bool UPDATE, int THREADS>
+ghb_status col_launch_batch_of(const ColItem* items, int n, int64_t blocks, size_t smem, int threads, cudaStream_t s) {
   static std::atomic<unsigned long long> mask{0};
-  TRY_STATUS(ensure_dyn_smem(rt_col_kernel_batch<SIGN, UPDATE>, 220 * 1024, mask));
-  return launch_chained(rt_col_kernel_batch<SIGN, UPDATE>, blocks, threads, smem, s, items, n);
+  TRY_STATUS(ensure_dyn_smem(rt_col_kernel_batch<SIGN, UPDATE, THREADS>, 220 * 1024, mask));
+  return launch_chained(rt_col_kernel_batch<SIGN, UPDATE, THREADS>, blocks, threads, smem, s, items, n);
+}
+template <int SIGN, bool UPDATE>
+ghb_status col_launch_batch(const ColItem* items, int n, int64_t blocks, size_t smem, int threads, cudaStream_t s) {
+  if (rt_many_warps(blocks, threads))
+    return col_launch_batch_of<SIGN, UPDATE, kRtManyThreads>(items, n, blocks, smem, threads, s);
+  return col_launch_batch_of<SIGN, UPDATE, kRtThreads>(items, n, blocks, smem, threads, s);
 }
 
 }  // namespace

@@ -19,11 +19,12 @@ def ghb():
     return g
 
 
-# double grids: groups of 2 .. 16 entries, padded and not, primes 7 .. 31, no pass, one pass, many passes
+# double grids: groups of 2 .. 16 entries, padded and not, primes 7 .. 31, no pass, one pass, many
+# passes, and enough warps for the kernels of 64 registers
 GRIDS = [((1, 1), (1, 1)), ((1, 3), (1, 5)), ((3, 5), (8, 9)), ((7, 7), (15, 16)), ((13, 15), (25, 31)), ((15, 31), (32, 64)),
          ((31, 33), (62, 77)), ((25, 63), (50, 125)), ((45, 99), (90, 198)), ((63, 127), (128, 256)), ((3, 481), (9, 961)),
          ((341, 3), (686, 5)), ((3, 1023), (5, 2048)), ((3, 3125), (5, 6250)), ((1023, 5), (2048, 9)),
-         ((3, 5, 7), (5, 9, 14)), ((15, 17, 33), (30, 34, 66)), ((33, 3, 41), (65, 7, 81))]
+         ((1023, 1023), (2048, 2048)), ((3, 5, 7), (5, 9, 14)), ((15, 17, 33), (30, 34, 66)), ((33, 3, 41), (65, 7, 81))]
 
 
 @pytest.mark.parametrize("N,M", GRIDS)
@@ -49,3 +50,21 @@ def test_operator_to_single_rounding(ghb, N, M, tile, rows):
     got, ref = ctx.matvec(x32).to(torch.complex128), ctx.matvec(x32.to(torch.complex128))
     tol = 4 * EPS * math.log2(max(math.prod(M), 2)) * math.sqrt(20.0)   # contrast 20: |A u| against |u|
     assert torch.linalg.norm(got - ref) <= tol * torch.linalg.norm(ref) + 1e-30
+
+
+@pytest.mark.parametrize("count", [1, 6])
+def test_batches_of_few_and_many_warps(ghb, count):
+    """One instance of N = 255 stays below the 24 warps an SM that choose the kernels
+    of 80 registers, six exceed them; either way the bounds are a single context's
+    to the solves' tolerance, which the energies meet squared."""
+    micros = [dict(d=2, N=[255, 255], a0=1.0, inclusions=[(1, (0.01 * i, -0.02 * i, 0.0), (0.31, 0.0, 0.0), 20.0 + i)])
+              for i in range(count)]
+    batch = ghb.Batch()
+    for m in micros:
+        batch.submit(m)
+    batch.run()
+    for m, r in zip(micros, sorted(batch.results(), key=lambda r: r["id"])):
+        upper, lower, _, status = ghb.Context.from_microstructure(m, precision="mixed").bounds()
+        assert status == 0
+        for got, want in ((r["upper"], upper), (r["lower"], lower)):
+            assert np.abs(np.asarray(got).reshape(2, 2) - want).max() <= 1e-10 * np.abs(want).max()

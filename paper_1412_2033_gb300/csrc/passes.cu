@@ -176,8 +176,9 @@ ghb_status launch_col<double>(int sign, int mode, const ColArgs& a, const FftPla
 template <>
 ghb_status launch_col<float>(int sign, int mode, const ColArgs& a, const FftPlan& pl, cudaStream_t s) {
   if (use_ct(pl, pl.ct_col != 0)) return launch_col_ct(sign, mode, a, pl, s);
-  if (a.outer * std::max<int64_t>(std::max(a.Lin, a.Lout), pl.M) * a.inner >= (int64_t(1) << 31)) {
-    set_error("column pass operand of 2^31 entries or more");
+  // the kernel's 32-bit offsets are row i times `inner` inside one outer index (RtColIn)
+  if (std::max<int64_t>(std::max(a.Lin, a.Lout), pl.M) * a.inner >= (int64_t(1) << 31)) {
+    set_error("column pass with 2^31 entries or more in one outer index");
     return GHB_ERR_INVALID;
   }
   int TW = pl.tile[1];   // ghb_tune_set; 0 = by the operand

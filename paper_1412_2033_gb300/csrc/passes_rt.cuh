@@ -106,7 +106,7 @@ struct RtColIn {
   const float2 *in, *old;
   float2* upd;
   float beta;
-  int inner;            // row stride (operands have fewer than 2^31 entries)
+  int inner;            // row stride (the rows of one outer index hold fewer than 2^31 entries)
   int half, wrap;       // rows: n <= half -> n + half, n >= wrap -> n - wrap (wrap = M - half)
   bool on;
   __device__ __forceinline__ int row(int n) const { return n <= half ? n + half : (n >= wrap ? n - wrap : -1); }

@@ -1,0 +1,102 @@
+"""What the pass launchers of csrc/passes.cu decide, on the host: the library's own
+dispatch code with recorders in place of the kernels' launchers."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_1412_2033_gb300", "csrc")
+
+RECORDERS = r"""
+#include <cstdio>
+#include <cstdlib>
+#include <cstring>
+#include "passes_fx.cuh"
+#include "passes_rt.cuh"
+namespace ghb {
+std::string error_text;
+int last_lines = 0, last_rows = 0, launched = 0;
+size_t last_smem = 0;
+void set_error(const std::string& s) { error_text = s; }
+ghb_status apply_tune(int, PlanHolder&) { return GHB_OK; }
+template <int M> ghb_status launch_col_ct_m(int, int, const ColArgs&, const CtTables&, cudaStream_t) { return GHB_OK; }
+template <int M> ghb_status launch_row_ct_m(int, const RowArgs&, const CtTables&, int, cudaStream_t) { return GHB_OK; }
+#define CT(m) template ghb_status launch_col_ct_m<m>(int, int, const ColArgs&, const CtTables&, cudaStream_t); \
+  template ghb_status launch_row_ct_m<m>(int, const RowArgs&, const CtTables&, int, cudaStream_t);
+CT(162) CT(486) CT(1458) CT(4374) CT(2187) CT(72) CT(135) CT(270)
+ghb_status col(const FxPlan& f, int TW, int eb) {
+  ++launched;
+  last_lines = TW;
+  last_smem = static_cast<size_t>(TW) * column_stride(f.ls, TW, eb) * eb;
+  return GHB_OK;
+}
+ghb_status row(const FxPlan& f, int rows, int lines, int eb) {
+  ++launched;
+  last_rows = rows;
+  last_lines = lines;
+  last_smem = static_cast<size_t>(lines) * f.ls * eb;
+  return GHB_OK;
+}
+ghb_status launch_fx_col(int, const ColArgs&, const FxPlan& f, int TW, cudaStream_t) { return col(f, TW, 16); }
+ghb_status launch_rt_col(int, const ColArgs&, const FxPlan& f, int TW, cudaStream_t) { return col(f, TW, 8); }
+ghb_status launch_fx_row(int, const RowArgs&, const FxPlan& f, int r, int n, int, cudaStream_t) { return row(f, r, n, 16); }
+ghb_status launch_rt_row(const RowArgs&, const FxPlan& f, int r, int n, cudaStream_t) { return row(f, r, n, 8); }
+ghb_status launch_fx_col_batch(int, const ColItem*, int, int64_t, size_t, int, cudaStream_t) { return GHB_OK; }
+ghb_status launch_rt_col_batch(int, bool, const ColItem*, int, int64_t, size_t, int, cudaStream_t) { return GHB_OK; }
+ghb_status launch_fx_row_batch(int, const RowItem*, int, int64_t, size_t, int, cudaStream_t) { return GHB_OK; }
+ghb_status launch_rt_row_batch(const RowItem*, int, int64_t, size_t, int, cudaStream_t) { return GHB_OK; }
+}  // namespace ghb
+using namespace ghb;
+"""
+
+
+@pytest.fixture(scope="module")
+def run(tmp_path_factory):
+    """run(body, *arguments): the words that main() { body } prints."""
+    tmp = tmp_path_factory.mktemp("launch_shapes")
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    flags = [nvcc, "-O2", "-std=c++17", "-w", "-gencode", "arch=compute_103a,code=sm_103a", "-I", CSRC, "-I",
+             os.path.join(ROOT, "include")]
+    objects = []
+    for unit in ("passes", "plan"):
+        objects.append(str(tmp / f"{unit}.o"))
+        subprocess.run([*flags, "-c", "-o", objects[-1], os.path.join(CSRC, unit + ".cu")], check=True)
+
+    def go(body, *arguments):
+        name = tmp / f"t{abs(hash(body))}"
+        (tmp / (name.name + ".cu")).write_text(RECORDERS + "int main(int argc, char** argv) {" + body + "}")
+        subprocess.run([*flags, "-o", str(name), str(name) + ".cu", *objects], check=True)
+        return subprocess.run([str(name), *map(str, arguments)], capture_output=True, text=True, check=True).stdout.split()
+
+    return go
+
+
+def test_column_offsets_are_bounded_by_one_outer_index(run):
+    """The FP32 column pass adds 32-bit row offsets to a 64-bit base: operands of 2^31
+    entries and more run as long as the rows of one outer index stay below (d = 3
+    axes at M = 1440 and 2560); beyond, the call is refused."""
+    out = run(r"""
+      auto ask = [](int64_t outer, int M, int N, int64_t inner) {
+        FftPlan p{};
+        group_plan(1, M, 32, p.rt, nullptr, nullptr);
+        p.M = M;
+        for (int sign : {+1, -1}) {
+          ColArgs a{};
+          a.outer = outer;
+          a.inner = inner;
+          a.Lin = sign > 0 ? N : M;
+          a.Lout = sign > 0 ? M : N;
+          launched = 0;
+          const ghb_status st = launch_col<float>(sign, COL_PLAIN, a, p, nullptr);
+          printf("%d%d ", st == GHB_OK, launched);
+        }
+      };
+      ask(3 * 1440, 1440, 715, 358);                    // axis 2 at N = 715: 2.2e9 entries
+      ask(3 * 2560LL, 2560, 1279, 640);                 // axis 2 at the largest order
+      ask(3, 2560, 1279, 1279LL * 640);                 // axis 1 there: 2095513600 entries an outer index
+      ask(1, 2048, 1023, (int64_t(1) << 31) / 2048 - 1);
+      ask(1, 2048, 1023, (int64_t(1) << 31) / 2048);    // 2^31 entries: refused
+    """)
+    assert out == ["11"] * 8 + ["00"] * 2

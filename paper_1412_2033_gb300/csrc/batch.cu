@@ -480,13 +480,15 @@ ghb_status prep_col(ghb_batch* b, int sign, int mode, std::vector<ColItem>& item
   // (their plans) are the tuned ones.
   // tiles of the flattened (outer, inner) range
   constexpr bool f64 = sizeof(T) == 8;
-  const int ls = longest_line<T>(b, Ms) + 15;   // column_stride of any item
-  const int TW = batch_lines<T>(ls);
+  const int TW = batch_lines<T>(longest_line<T>(b, Ms) + 15);
+  auto stride = [&](int M, int tile) { return column_stride(line_length<T>(b, M), tile, 2 * sizeof(T)); };
+  int ls = 1;
+  for (int M : Ms) ls = std::max(ls, stride(M, TW));
   int64_t blocks = 0;
   for (size_t i = 0; i < items.size(); ++i) {
     ColItem& it = items[i];
     it.tile = TW;
-    while (it.tile < 32 && 2 * it.tile * (line_length<T>(b, Ms[i]) + 15) <= TW * ls) it.tile *= 2;
+    while (it.tile < 32 && 2 * it.tile * stride(Ms[i], 2 * it.tile) <= TW * ls) it.tile *= 2;
     it.block_begin = blocks;
     blocks += (it.a.inner * it.a.outer + it.tile - 1) / it.tile;
   }

@@ -298,8 +298,13 @@ FX_HD int fx_tracked(int lo, int hi) { return hi > ~lo ? hi : ~lo; }   // lo <= 
 struct UnitRoot {
   long double c, s;   // cos, sin of 2 pi j / M
 };
-// (perm_out, nat_out: the tables of FxPlan, left out when null)
-bool group_plan(int k, int M, int cap, FxPlan& f, std::vector<int>* perm_out, std::vector<int>* nat_out);
+// (perm_out, nat_out: the tables of FxPlan, left out when null).  Spare positions are
+// left out as far as the line then takes at most max_ls positions.
+bool group_plan(int k, int M, int cap, FxPlan& f, std::vector<int>* perm_out, std::vector<int>* nat_out,
+                int max_ls = 1 << 30);
+// The most positions a line of length M may take for every launch that admits M to
+// fit a CTA's shared memory, `tile` columns a CTA among them.
+int line_limit(int k, int M, int tile);
 void unit_roots(int M, std::vector<UnitRoot>& r);
 void fx_twiddles(const std::vector<UnitRoot>& roots, std::vector<fxw>& tw);
 

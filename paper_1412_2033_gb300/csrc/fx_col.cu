@@ -24,7 +24,7 @@ namespace {
 template <int SIGN>
 ghb_status col_launch(const ColArgs& a, const FxPlan& f, int TW, cudaStream_t s) {
   static std::atomic<unsigned long long> mask{0};
-  TRY_STATUS(ensure_dyn_smem(fx_col_kernel<SIGN>, 220 * 1024, mask));
+  TRY_STATUS(ensure_dyn_smem(fx_col_kernel<SIGN>, kPassSmem, mask));
   const size_t smem = static_cast<size_t>(TW) * column_stride(f.ls, TW, sizeof(fx2)) * sizeof(fx2);
   const int64_t grid = (a.outer * a.inner + TW - 1) / TW;
   return launch_chained(fx_col_kernel<SIGN>, grid, fx_threads(f.M, TW, f.ls), smem, s, a, f, TW);
@@ -34,7 +34,7 @@ template <int SIGN>
 ghb_status col_launch_batch(const ColItem* items, int n, int64_t blocks, size_t smem, int threads,
                             cudaStream_t s) {
   static std::atomic<unsigned long long> mask{0};
-  TRY_STATUS(ensure_dyn_smem(fx_col_kernel_batch<SIGN>, 220 * 1024, mask));
+  TRY_STATUS(ensure_dyn_smem(fx_col_kernel_batch<SIGN>, kPassSmem, mask));
   return launch_chained(fx_col_kernel_batch<SIGN>, blocks, threads, smem, s, items, n);
 }
 

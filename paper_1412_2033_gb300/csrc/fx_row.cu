@@ -24,7 +24,7 @@ namespace {
 template <int MODE>
 ghb_status row_launch(const RowArgs& a, const FxPlan& f, int rows_per_cta, int NL, int threads, cudaStream_t s) {
   static std::atomic<unsigned long long> mask{0};
-  TRY_STATUS(ensure_dyn_smem(fx_row_kernel<MODE>, 220 * 1024, mask));
+  TRY_STATUS(ensure_dyn_smem(fx_row_kernel<MODE>, kPassSmem, mask));
   const size_t smem = static_cast<size_t>(NL) * f.ls * sizeof(fx2);
   int64_t grid = (a.rows + rows_per_cta - 1) / rows_per_cta;
   if (MODE == ROW_ENERGY && grid > 1024) grid = 1024;   // partials hold 1024 x 6 doubles
@@ -35,7 +35,7 @@ template <int MODE>
 ghb_status row_launch_batch(const RowItem* items, int n, int64_t blocks, size_t smem, int threads,
                             cudaStream_t s) {
   static std::atomic<unsigned long long> mask{0};
-  TRY_STATUS(ensure_dyn_smem(fx_row_kernel_batch<MODE>, 220 * 1024, mask));
+  TRY_STATUS(ensure_dyn_smem(fx_row_kernel_batch<MODE>, kPassSmem, mask));
   return launch_chained(fx_row_kernel_batch<MODE>, blocks, threads, smem, s, items, n);
 }
 

@@ -121,9 +121,10 @@ struct PlanHolder {
 ghb_status make_plan(int M, PlanHolder& out);
 ghb_status make_plan_untuned(int M, PlanHolder& out);
 // Regroup the transform of precision k ([0] FP64, [1] FP32) into passes of group
-// size <= cap (5 at least) and replace its digit-reversal table on the device.
+// size <= cap (5 at least), with lines that fit `tile` columns a CTA, and replace its
+// digit-reversal table on the device.
 constexpr int kGroupCap[2] = {18, 32};
-ghb_status set_group_cap(PlanHolder& h, int k, int cap);
+ghb_status set_group_cap(PlanHolder& h, int k, int cap, int tile);
 // Write the autotuned configuration for length M into p (tuning M first if
 // it has not been tuned in this process and tuning is enabled).
 ghb_status apply_tune(int M, PlanHolder& h);
@@ -349,6 +350,13 @@ __host__ __device__ constexpr size_t col_smem_bytes(int M, int TW, int elem_byte
   return elem_bytes == 8 ? padded_elems<float2>(static_cast<size_t>(M) * TW) * 8
                          : padded_elems<double2>(static_cast<size_t>(M) * TW) * 16;
 }
+// Dynamic shared memory that the run-time passes may take, and the sizes that they
+// admit: `tile` columns a CTA, `lines` complex lines of a last-axis pass.  The rules
+// count one spare entry every 128 bytes; the lines' own layouts hold theirs elsewhere
+// and leave them out where they would not fit (line_limit, plan.cu).
+constexpr size_t kPassSmem = 220 * 1024;
+inline bool col_admitted(int M, int tile, int elem_bytes) { return col_smem_bytes(M, tile, elem_bytes) <= kPassSmem; }
+inline bool row_admitted(int M, int lines, int elem_bytes) { return col_smem_bytes(M, lines, elem_bytes) <= 200 * 1024; }
 __host__ __device__ constexpr int col_tile_width(int M, int elem_bytes) {
   const size_t budget = 160 * 1024;
   for (int tw : {16, 8, 4, 2}) {

@@ -131,7 +131,7 @@ int rt_col_tile(int M, int ls, int64_t columns) {
     const int64_t ctas = (columns + tw - 1) / tw;
     if (smem <= (tw == 4 ? 150 : 73) * 1024 && 10 * ctas >= (tw == 4 ? 16 : 20) * device_sms()) return tw;
   }
-  return 2;
+  return 2 * column_stride(ls, 2, sizeof(float2)) * sizeof(float2) <= kPassSmem ? 2 : 1;
 }
 // More warps than the 24 that kernels of 80 registers keep on every SM.
 bool rt_many_warps(int64_t blocks, int threads) {
@@ -162,9 +162,8 @@ void rt_row_shape(int ncomp, int M, int ls, int64_t rows, int want, int* rows_pe
 template <>
 ghb_status launch_col<double>(int sign, int mode, const ColArgs& a, const FftPlan& pl, cudaStream_t s) {
   int TW = pl.tile[0];   // ghb_tune_set; 0 = by the operand
-  if (TW <= 0 || static_cast<size_t>(TW) * (pl.fx.ls + 15) * sizeof(fx2) > 220 * 1024)
-    TW = fx_col_tile(pl.fx.ls, a.outer * a.inner);
-  if (col_smem_bytes(pl.M, 1, sizeof(double2)) > 220 * 1024) {
+  if (TW <= 0) TW = fx_col_tile(pl.fx.ls, a.outer * a.inner);
+  if (!col_admitted(pl.M, 1, sizeof(double2))) {
     set_error("transform length too large for one CTA: M=" + std::to_string(pl.M));
     return GHB_ERR_INVALID;
   }
@@ -182,8 +181,11 @@ ghb_status launch_col<float>(int sign, int mode, const ColArgs& a, const FftPlan
     return GHB_ERR_INVALID;
   }
   int TW = pl.tile[1];   // ghb_tune_set; 0 = by the operand
-  if (TW <= 0 || static_cast<size_t>(TW) * (pl.rt.ls + 15) * sizeof(float2) > 220 * 1024)
-    TW = rt_col_tile(pl.M, pl.rt.ls, a.outer * a.inner);
+  if (TW <= 0) TW = rt_col_tile(pl.M, pl.rt.ls, a.outer * a.inner);
+  if (!col_admitted(pl.M, 1, sizeof(float2))) {
+    set_error("transform length too large for one CTA: M=" + std::to_string(pl.M));
+    return GHB_ERR_INVALID;
+  }
   ColArgs b = a;
   if (mode != COL_PUPDATE) b.pold = nullptr;
   return launch_rt_col(sign, b, pl.rt, TW, s);
@@ -231,6 +233,10 @@ ghb_status launch_row<float>(int mode, const RowArgs& a, const FftPlan& pl, cuda
   row_lines(mode, a.nfields, a.ncomp, pl.M, pl.rows32, &rows_per_cta, &NL);
   if (mode == ROW_MATVEC) {   // set-up and Gram passes run in FP64 only
     if (use_ct(pl, pl.ct_row != 0)) return launch_row_ct(NL, a, pl, rows_per_cta, s);
+    if (!row_admitted(pl.M, NL, sizeof(float2))) {
+      set_error("row transform too large for one CTA: M=" + std::to_string(pl.M));
+      return GHB_ERR_INVALID;
+    }
     int lines = 1;
     rt_row_shape(a.ncomp, pl.M, pl.rt.ls, a.rows, pl.rows32, &rows_per_cta, &lines);
     return launch_rt_row(a, pl.rt, rows_per_cta, lines, s);
@@ -243,7 +249,7 @@ template <>
 ghb_status launch_row<double>(int mode, const RowArgs& a, const FftPlan& pl, cudaStream_t s) {
   int rows_per_cta = 1, NL = 1, threads = 256;
   row_lines(mode, a.nfields, a.ncomp, pl.M, 0, &rows_per_cta, &NL);
-  if (padded_elems<double2>(static_cast<size_t>(pl.M) * NL) * sizeof(double2) > 200 * 1024) {
+  if (!row_admitted(pl.M, NL, sizeof(double2))) {
     set_error("row transform too large for one CTA: M=" + std::to_string(pl.M));
     return GHB_ERR_INVALID;
   }

@@ -74,7 +74,7 @@ struct Cover {
 // Passes of a run-time transform (k = 0: fft_fx.cuh, 1: fft_rt.cuh): as few as the
 // cap allows, odd group sizes first (the first pass's threads then sit at an odd
 // stride), primes above 5 last.
-bool group_plan(int k, int M, int cap, FxPlan& f, std::vector<int>* perm_out, std::vector<int>* nat_out) {
+bool group_plan(int k, int M, int cap, FxPlan& f, std::vector<int>* perm_out, std::vector<int>* nat_out, int max_ls) {
   f.M = M;
   int a = 0, b = 0, c = 0, m = M;
   while (m % 2 == 0) { ++a; m /= 2; }
@@ -121,6 +121,7 @@ bool group_plan(int k, int M, int cap, FxPlan& f, std::vector<int>* perm_out, st
     L *= p.size();
     if (L < M && L >= 8 && position(L) % 4 == 0) spare.push_back(L);
   }
+  while (!spare.empty() && position(M - 1) + 1 > max_ls) spare.pop_back();
   f.ls = M > 0 ? position(M - 1) + 1 : 1;
   int lp = 1;
   std::vector<int> radix;
@@ -184,6 +185,18 @@ bool group_plan(int k, int M, int cap, FxPlan& f, std::vector<int>* perm_out, st
     for (int n = 0; n < M; ++n) (*nat_out)[n] = position(n);
   }
   return true;
+}
+
+int line_limit(int k, int M, int tile) {
+  const int eb = k == 0 ? 16 : 8;
+  const int T = tile > 1 ? tile : 1;
+  // column_stride rounds a line up to `want` modulo `period`
+  const int period = 128 / eb, want = T < period ? period / T : 1;
+  const int most = static_cast<int>(kPassSmem / (static_cast<size_t>(T) * eb));
+  int limit = most - ((most - want) & (period - 1));
+  for (int lines = 1; lines <= 5; ++lines)
+    if (row_admitted(M, lines, eb)) limit = std::min(limit, static_cast<int>(kPassSmem / (static_cast<size_t>(lines) * eb)));
+  return limit;
 }
 
 // cos and sin of 2 pi j / M for j = 0 .. M-1, each evaluated at an angle of the
@@ -258,8 +271,8 @@ ghb_status build_plan_tables(int M, FftPlan& p, PlanTables& t) {
   }
   p = FftPlan{};
   p.M = M;
-  if (!group_plan(0, M, kGroupCap[0], p.fx, &t.perm_of[0], &t.nat_of[0]) ||
-      !group_plan(1, M, kGroupCap[1], p.rt, &t.perm_of[1], &t.nat_of[1])) {
+  if (!group_plan(0, M, kGroupCap[0], p.fx, &t.perm_of[0], &t.nat_of[0], line_limit(0, M, 1)) ||
+      !group_plan(1, M, kGroupCap[1], p.rt, &t.perm_of[1], &t.nat_of[1], line_limit(1, M, 1))) {
     set_error("internal: no passes for M=" + std::to_string(M));
     return GHB_ERR_INVALID;
   }
@@ -281,11 +294,11 @@ ghb_status make_plan(int M, PlanHolder& out) {
   return apply_tune(M, out);
 }
 
-ghb_status set_group_cap(PlanHolder& out, int k, int cap) {
+ghb_status set_group_cap(PlanHolder& out, int k, int cap, int tile) {
   FftPlan& p = out.plan;
   FxPlan f = k == 0 ? p.fx : p.rt;
   std::vector<int> perm, nat;
-  if (!group_plan(k, p.M, cap, f, &perm, &nat)) {
+  if (!group_plan(k, p.M, cap, f, &perm, &nat, line_limit(k, p.M, tile))) {
     set_error("internal: no passes for M=" + std::to_string(p.M));
     return GHB_ERR_INVALID;
   }

@@ -24,7 +24,7 @@ namespace {
 template <int SIGN, bool UPDATE>
 ghb_status col_launch(const ColArgs& a, const FxPlan& f, int TW, cudaStream_t s) {
   static std::atomic<unsigned long long> mask{0};
-  TRY_STATUS(ensure_dyn_smem(rt_col_kernel<SIGN, UPDATE>, 220 * 1024, mask));
+  TRY_STATUS(ensure_dyn_smem(rt_col_kernel<SIGN, UPDATE>, kPassSmem, mask));
   const size_t smem = static_cast<size_t>(TW) * column_stride(f.ls, TW, sizeof(float2)) * sizeof(float2);
   const int64_t grid = (a.outer * a.inner + TW - 1) / TW;
   return launch_chained(rt_col_kernel<SIGN, UPDATE>, grid, rt_threads(f.M, TW, f.ls), smem, s, a, f, TW);
@@ -33,7 +33,7 @@ ghb_status col_launch(const ColArgs& a, const FxPlan& f, int TW, cudaStream_t s)
 template <int SIGN, bool UPDATE, int THREADS>
 ghb_status col_launch_batch_of(const ColItem* items, int n, int64_t blocks, size_t smem, int threads, cudaStream_t s) {
   static std::atomic<unsigned long long> mask{0};
-  TRY_STATUS(ensure_dyn_smem(rt_col_kernel_batch<SIGN, UPDATE, THREADS>, 220 * 1024, mask));
+  TRY_STATUS(ensure_dyn_smem(rt_col_kernel_batch<SIGN, UPDATE, THREADS>, kPassSmem, mask));
   return launch_chained(rt_col_kernel_batch<SIGN, UPDATE, THREADS>, blocks, threads, smem, s, items, n);
 }
 template <int SIGN, bool UPDATE>

@@ -25,7 +25,7 @@ template <int THREADS>
 ghb_status row_launch(const RowArgs& a, const FxPlan& f, int64_t grid, int threads, int rows_per_cta, int lines,
                       cudaStream_t s) {
   static std::atomic<unsigned long long> mask{0};
-  TRY_STATUS(ensure_dyn_smem(rt_row_kernel<THREADS>, 200 * 1024, mask));
+  TRY_STATUS(ensure_dyn_smem(rt_row_kernel<THREADS>, kPassSmem, mask));
   const size_t smem = static_cast<size_t>(lines) * f.ls * sizeof(float2);
   return launch_chained(rt_row_kernel<THREADS>, grid, threads, smem, s, a, f, rows_per_cta, lines);
 }
@@ -33,7 +33,7 @@ ghb_status row_launch(const RowArgs& a, const FxPlan& f, int64_t grid, int threa
 template <int THREADS>
 ghb_status row_launch_batch(const RowItem* items, int n, int64_t blocks, size_t smem, int threads, cudaStream_t s) {
   static std::atomic<unsigned long long> mask{0};
-  TRY_STATUS(ensure_dyn_smem(rt_row_kernel_batch<THREADS>, 200 * 1024, mask));
+  TRY_STATUS(ensure_dyn_smem(rt_row_kernel_batch<THREADS>, kPassSmem, mask));
   return launch_chained(rt_row_kernel_batch<THREADS>, blocks, threads, smem, s, items, n);
 }
 

@@ -30,6 +30,7 @@
 #include <map>
 #include <mutex>
 
+#include "fft_fx.cuh"
 #include "ghb_internal.cuh"
 
 namespace ghb {
@@ -60,10 +61,10 @@ Tune size_rules(int M) {
 
 ghb_status write_tune(const Tune& t, PlanHolder& h) {
   FftPlan& p = h.plan;
-  const int caps[2] = {t.cap64, t.cap32};
+  const int caps[2] = {t.cap64, t.cap32}, tiles[2] = {t.tile64, t.tile32};
   for (int k = 0; k < 2; ++k)
-    if (h.cap[k] != caps[k]) {
-      const ghb_status st = set_group_cap(h, k, caps[k]);
+    if (h.cap[k] != caps[k] || (k == 0 ? p.fx.ls : p.rt.ls) > line_limit(k, p.M, tiles[k])) {
+      const ghb_status st = set_group_cap(h, k, caps[k], tiles[k]);
       if (st != GHB_OK) return st;
     }
   p.tile[1] = t.tile32;
@@ -259,7 +260,7 @@ ghb_status tune_length(int M, Tune* out) {
     args(false, inv, fwd, row);
     float best_total = 1e30f;
     for (int cap : {9, 18}) {
-      TUNE_TRY(set_group_cap(ph, 0, cap));
+      TUNE_TRY(set_group_cap(ph, 0, cap, 1));
       FftPlan p = ph.plan;
       float col_best = 1e30f;
       {
@@ -286,7 +287,7 @@ bool valid_tune(int M, const Tune& t) {
   const bool caps = t.cap32 >= 5 && t.cap32 <= 32 && t.cap64 >= 5 && t.cap64 <= 32;
   auto tile_ok = [&](int tile, int eb) {
     return tile == 0 || ((tile == 1 || tile == 2 || tile == 4 || tile == 8 || tile == 16) &&
-                         col_smem_bytes(M, tile, eb) <= 220 * 1024);
+                         col_admitted(M, tile, eb));
   };
   const bool rows = t.rows32 >= 0 && t.rows32 <= 2;
   const bool ct = (t.ct_col == 0 || t.ct_col == 1) && (t.ct_row == 0 || t.ct_row == 1) &&

@@ -100,3 +100,70 @@ def test_column_offsets_are_bounded_by_one_outer_index(run):
       ask(1, 2048, 1023, (int64_t(1) << 31) / 2048);    // 2^31 entries: refused
     """)
     assert out == ["11"] * 8 + ["00"] * 2
+
+
+def test_every_admitted_length_and_tile_fits_shared_memory(run):
+    """Lengths with primes up to 31, every group size: what the size rules admit
+    (columns of one line, forced tiles, rows) is launched as asked, in the kernels'
+    220 KB, and with lines whose entries are evenly spaced in every group.  One length
+    more than that is refused with a message."""
+    out = run(r"""
+      int bad = 0, dropped = 0, launches = 0;
+      for (int M = 1; M <= 27000; ++M) {
+        if (!factorizable(M)) continue;
+        for (int k = 0; k < 2; ++k)
+          for (int cap : {5, 8, 9, 10, 16, 32}) {
+            const int eb = k == 0 ? 16 : 8;
+            FftPlan p{};
+            p.M = M;
+            FxPlan& f = k == 0 ? p.fx : p.rt;
+            std::vector<int> pos;
+            for (int tile : {0, 1, 2, 4, 8, 16}) {
+              if (tile == 0) group_plan(k, M, cap, f, nullptr, nullptr, line_limit(k, M, 1));
+              if (tile > 0 && !col_admitted(M, tile, eb)) continue;
+              if (f.ls > line_limit(k, M, tile)) {     // as tune.cu does for a forced tile
+                ++dropped;
+                group_plan(k, M, cap, f, nullptr, &pos, line_limit(k, M, tile));
+                std::vector<char> seen(f.ls, 0);
+                for (int n = 0; n < M; ++n) bad += pos[n] < 0 || pos[n] >= f.ls || seen[pos[n]]++;
+                for (int i = 0; i < f.np; ++i)
+                  for (int u = 0, q; u < f.p[i].units; ++u)
+                    for (int j = 0, e = fx_unit_entry(f.p[i], u, q); j < f.p[i].R; ++j)
+                      bad += pos[e] + j * f.p[i].step != pos[e + j * f.p[i].lp];
+              }
+              p.tile[k] = tile;
+              for (int64_t columns : {1, 50000}) {
+                ColArgs a{};
+                a.outer = 1;
+                a.inner = columns;
+                a.Lin = M;
+                a.Lout = M;
+                launched = 0;
+                const ghb_status st = k == 0 ? launch_col<double>(-1, COL_PLAIN, a, p, nullptr) : launch_col<float>(-1, COL_PLAIN, a, p, nullptr);
+                launches += launched;
+                if (!col_admitted(M, 1, eb)) bad += st == GHB_OK || launched || error_text.find("too large") == std::string::npos;
+                else bad += st != GHB_OK || launched != 1 || last_smem > kPassSmem || (tile > 0 && last_lines != tile);
+              }
+            }
+            group_plan(k, M, cap, f, nullptr, nullptr, line_limit(k, M, 1));
+            for (int d : {2, 3})
+              for (int mode : {ROW_MATVEC, ROW_TOREAL, ROW_ENERGY})
+                for (int64_t rows : {1, 5, 100000}) {
+                  if (k == 1 && mode != ROW_MATVEC) continue;
+                  RowArgs a{};
+                  a.nfields = mode == ROW_ENERGY ? d : 1;
+                  a.ncomp = mode == ROW_TOREAL ? 1 : d;
+                  a.rows = rows;
+                  int r, n;
+                  row_lines(mode, a.nfields, a.ncomp, M, 0, &r, &n);
+                  launched = 0;
+                  const ghb_status st = k == 0 ? launch_row<double>(mode, a, p, nullptr) : launch_row<float>(mode, a, p, nullptr);
+                  launches += launched;
+                  if (!row_admitted(M, n, eb)) bad += st == GHB_OK || launched || error_text.find("too large") == std::string::npos;
+                  else bad += st != GHB_OK || launched != 1 || last_smem > kPassSmem;
+                }
+          }
+      }
+      printf("%d %d %d", bad, dropped > 100, launches > 100000);
+    """)
+    assert out == ["0", "1", "1"]

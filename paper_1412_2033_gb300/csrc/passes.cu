@@ -146,10 +146,12 @@ int rt_threads(int M, int lines, int ls) {
 }
 // Last axis: the least rows that fill complex lines (d = 2: one, d = 3: two rows,
 // three lines), doubled while a block of 256 has threads without a group and two
-// CTAs remain for each SM; `want` = 1 keeps the least, 2 doubles it once.
+// CTAs remain for each SM; `want` = 1 keeps the least, 2 doubles it once (d = 2:
+// at every length whose two lines are admitted, as ghb_tune_set promises).
 void rt_row_shape(int ncomp, int M, int ls, int64_t rows, int want, int* rows_per_cta, int* lines) {
   int r = ncomp == 2 ? 1 : 2, q = r * ncomp / 2;
-  while (want != 1 && 2 * q <= kRtMaxLines && static_cast<size_t>(2 * q) * ls * sizeof(float2) <= 73 * 1024 &&
+  const size_t most = want == 2 && ncomp == 2 ? kPassSmem : 73 * 1024;
+  while (want != 1 && 2 * q <= kRtMaxLines && static_cast<size_t>(2 * q) * ls * sizeof(float2) <= most &&
          (want == 2 || (q * (M / 16) < 192 && rows / (2 * r) >= 2 * device_sms()))) {
     r *= 2;
     q *= 2;

@@ -167,3 +167,28 @@ def test_every_admitted_length_and_tile_fits_shared_memory(run):
       printf("%d %d %d", bad, dropped > 100, launches > 100000);
     """)
     assert out == ["0", "1", "1"]
+
+
+def test_forced_rows_are_launched(run):
+    """rows32 of ghb_tune_set is what a d = 2 FP32 last-axis pass launches, at every
+    length whose two lines are admitted."""
+    out = run(r"""
+      int bad = 0, n = 0;
+      for (int M = 1; M <= 13000; ++M) {
+        if (!factorizable(M) || !row_admitted(M, 2, 8)) continue;
+        FftPlan p{};
+        p.M = M;
+        group_plan(1, M, 32, p.rt, nullptr, nullptr, line_limit(1, M, 1));
+        for (int rows : {1, 2}) {
+          p.rows32 = rows;
+          RowArgs a{};
+          a.nfields = 1;
+          a.ncomp = 2;
+          a.rows = 100;
+          bad += launch_row<float>(ROW_MATVEC, a, p, nullptr) != GHB_OK || last_rows != rows || last_smem > kPassSmem;
+          ++n;
+        }
+      }
+      printf("%d %d", bad, n > 1000);
+    """)
+    assert out == ["0", "1"]

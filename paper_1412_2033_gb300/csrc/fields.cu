@@ -477,23 +477,23 @@ __device__ void op_init(const CgItem& it, int64_t bid, int64_t nb) {
   C* p = static_cast<C*>(it.p);
   const C* b = static_cast<const C*>(it.b);
   CgState* st = it.st;
-  // per-thread partial sums in the field's precision (a few dozen terms), the
-  // cross-thread and cross-block sums in FP64
-  T acc = T(0);
+  ThreadSum<T> acc;   // the cross-thread and cross-block sums in FP64
   GHB_FIELD_LOOP(e, fg, bid, nb) {
     const int j = jindex(fg, e);
     const T wt = (j == 0) ? T(1) : T(2);
+    T sacc = acc.open();
     for (int c = 0; c < fg.d; ++c) {
       const int64_t i = c * fg.P + e;
       const C bv = b[i];
       x[i] = mk(T(0), T(0));
       p[i] = mk(T(0), T(0));
       r[i] = bv;
-      acc += wt * (bv.x * bv.x + bv.y * bv.y);
+      sacc += wt * (bv.x * bv.x + bv.y * bv.y);
     }
+    acc.close(sacc);
   }
   double tot;
-  if (grid_sum_last(static_cast<double>(acc), it.partials, &st->ticket, &tot, bid, nb)) {
+  if (grid_sum_last(acc.total(), it.partials, &st->ticket, &tot, bid, nb)) {
     st->bb = tot;
     st->rr = tot;
     st->tol2 = it.tol * it.tol * tot;
@@ -509,15 +509,15 @@ __device__ void op_init(const CgItem& it, int64_t bid, int64_t nb) {
 }
 
 // Per-thread part of op_project_dot: q = G w on this thread's entries and
-// their share of <p, q> (in the field's precision).
+// their share of <p, q>.
 template <typename T, int D>
-__device__ __forceinline__ T project_dot_loop(const CgItem& it, int64_t bid, int64_t nb) {
+__device__ __forceinline__ double project_dot_loop(const CgItem& it, int64_t bid, int64_t nb) {
   using C = typename CT<T>::type;
   const FieldGeom& fg = it.fg;
   C* q = static_cast<C*>(it.q);
   const C* w = static_cast<const C*>(it.w);
   const C* p = static_cast<const C*>(it.p);
-  T acc = T(0);
+  ThreadSum<T> acc;
   GHB_FIELD_LOOP(e, fg, bid, nb) {
     int k[3];
     int j;
@@ -537,9 +537,9 @@ __device__ __forceinline__ T project_dot_loop(const CgItem& it, int64_t bid, int
       q[c * fg.P + e] = qv[c];
       sacc += pv[c].x * qv[c].x + pv[c].y * qv[c].y;
     }
-    acc += wt * sacc;
+    acc.close(acc.open() + wt * sacc);
   }
-  return acc;
+  return acc.total();
 }
 
 // q = G w, <p, q>; the last block forms alpha = <r, r> / <p, A p>.
@@ -548,9 +548,9 @@ __device__ void op_project_dot(const CgItem& it, int64_t bid, int64_t nb) {
   const FieldGeom& fg = it.fg;
   CgState* st = it.st;
   if (st->done != RUNNING) return;
-  const T acc = fg.d == 2 ? project_dot_loop<T, 2>(it, bid, nb) : project_dot_loop<T, 3>(it, bid, nb);
+  const double acc = fg.d == 2 ? project_dot_loop<T, 2>(it, bid, nb) : project_dot_loop<T, 3>(it, bid, nb);
   double tot;
-  if (grid_sum_last(static_cast<double>(acc), it.partials, &st->ticket, &tot, bid, nb)) {
+  if (grid_sum_last(acc, it.partials, &st->ticket, &tot, bid, nb)) {
     st->pq = tot;
     if (!(tot > 0.0) || !isfinite(tot)) {
       st->done = BREAKDOWN;
@@ -564,17 +564,18 @@ __device__ void op_project_dot(const CgItem& it, int64_t bid, int64_t nb) {
 // Per-thread part of op_update: x += alpha p, r -= alpha q on this thread's
 // entries and their share of <r, r>.
 template <typename T, int D>
-__device__ __forceinline__ T update_loop(const CgItem& it, T al, int64_t bid, int64_t nb) {
+__device__ __forceinline__ double update_loop(const CgItem& it, T al, int64_t bid, int64_t nb) {
   using C = typename CT<T>::type;
   const FieldGeom& fg = it.fg;
   C* x = static_cast<C*>(it.x);
   C* r = static_cast<C*>(it.r);
   const C* p = static_cast<const C*>(it.p);
   const C* q = static_cast<const C*>(it.q);
-  T acc = T(0);
+  ThreadSum<T> acc;
   GHB_FIELD_LOOP(e, fg, bid, nb) {
     const int j = jindex(fg, e);
     const T wt = (j == 0) ? T(1) : T(2);
+    T sacc = acc.open();
     C pv[D], qv[D], xv[D], rv[D];
 #pragma unroll
     for (int c = 0; c < D; ++c) {
@@ -591,10 +592,11 @@ __device__ __forceinline__ T update_loop(const CgItem& it, T al, int64_t bid, in
       const C rn = mk(rv[c].x - al * qv[c].x, rv[c].y - al * qv[c].y);
       x[i] = xn;
       r[i] = rn;
-      acc += wt * (rn.x * rn.x + rn.y * rn.y);
+      sacc += wt * (rn.x * rn.x + rn.y * rn.y);
     }
+    acc.close(sacc);
   }
-  return acc;
+  return acc.total();
 }
 
 // x += alpha p, r -= alpha q, <r, r>; the last block forms beta and the stop test.
@@ -604,10 +606,9 @@ __device__ void op_update(const CgItem& it, int64_t bid, int64_t nb) {
   CgState* st = it.st;
   if (st->done != RUNNING) return;
   const T al = static_cast<T>(st->alpha);
-  // per-thread partial in the field's precision, FP64 across threads
-  const T acc = fg.d == 2 ? update_loop<T, 2>(it, al, bid, nb) : update_loop<T, 3>(it, al, bid, nb);
+  const double acc = fg.d == 2 ? update_loop<T, 2>(it, al, bid, nb) : update_loop<T, 3>(it, al, bid, nb);
   double tot;
-  if (grid_sum_last(static_cast<double>(acc), it.partials, &st->ticket, &tot, bid, nb)) {
+  if (grid_sum_last(acc, it.partials, &st->ticket, &tot, bid, nb)) {
     const double rr_old = st->rr;
     st->beta = tot / rr_old;
     st->rr = tot;

@@ -419,14 +419,17 @@ CgItem cg_item(const Slot& s) {
 template <typename T>
 ghb_status prep_cg(ghb_batch* b, int op, std::vector<CgItem>& items, std::vector<Launch>& out) {
   if (items.empty()) return GHB_OK;
-  // About one wave of blocks in all, up to eight entries a thread: a block ends in
-  // a reduction of 45 FP64 instructions a warp, which kept the FP64 pipe busy for
-  // most of the launch at one entry a thread (256 solves of N = 31 ..
-  // 255: update 49 -> 29 us, projection 46 -> 23 us a launch).
-  int64_t blocks = 0, all = 0;
-  for (const auto& it : items) all += it.nblocks;
-  const int64_t each = std::min<int64_t>(std::max<int64_t>(all / 1216, 1), 8);
+  // Entries a thread: a block ends in a reduction on the FP64 pipe (12 instructions) and
+  // a ticket, which for many solves cost more than the entries; for few, a thread's
+  // entries one after the other cost more.  The split goes by the item's own size (one
+  // below 2048 entries, two below 10240, four from there), not by the launch's, so that
+  // its sums, and with them its bounds, are the same alone and beside other requests.
+  // Measured (ms; one for all, four for all, this rule): 64 mixed microstructures of
+  // N = 31 .. 255 82 / 73.9 / 74.1, 256 of N = 31 .. 127 159 / 146 / 150, 23 of N = 31 .. 77
+  // 11.0 / 11.4 / 11.1, two of N = 127 4.29 / 4.47 / 4.29.
+  int64_t blocks = 0;
   for (auto& it : items) {
+    const int64_t each = it.nblocks < 8 ? 1 : (it.nblocks < 40 ? 2 : 4);
     it.nblocks = (it.nblocks + each - 1) / each;
     it.block_begin = blocks;
     blocks += it.nblocks;

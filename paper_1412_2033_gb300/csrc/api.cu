@@ -950,7 +950,7 @@ ghb_status alloc_ctx(ghb_ctx* c) {
 ghb_status ensure_planN(ghb_ctx* c) {
   const Geometry& g = c->g;
   const int d = g.d;
-  if (c->planN[c->planN_of_axis[0]].d_tw32 != nullptr) return GHB_OK;
+  if (c->planN[c->planN_of_axis[0]].d_tables != nullptr) return GHB_OK;
   for (int a = 0; a < d; ++a)
     if (!factorizable(g.N[a])) {
       set_error("the N-grid transforms have length N; N=" + std::to_string(g.N[a]) +

@@ -107,11 +107,9 @@ struct Geometry {
 // Host-owned plan with its device tables.
 struct PlanHolder {
   FftPlan plan{};
-  int* d_perm_ct = nullptr;
-  float2* d_tw32 = nullptr;
-  fxw* d_fx_tw = nullptr;
-  // digit reversal and positions (perm, then nat) and group-size cap of the
-  // transforms' current groupings ([0] FP64, [1] FP32)
+  char* d_tables = nullptr;   // one allocation holds all of them
+  // in it: digit reversal and positions (perm, then nat) of the transforms' current
+  // groupings ([0] FP64, [1] FP32), and the groupings' size caps
   int* d_group_perm[2] = {nullptr, nullptr};
   int cap[2] = {0, 0};
 };

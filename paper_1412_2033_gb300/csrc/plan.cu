@@ -2,6 +2,7 @@
 #include <algorithm>
 #include <climits>
 #include <cmath>
+#include <cstring>
 #include <vector>
 
 #include "fft_ct.cuh"
@@ -302,8 +303,8 @@ ghb_status set_group_cap(PlanHolder& out, int k, int cap, int tile) {
     set_error("internal: no passes for M=" + std::to_string(p.M));
     return GHB_ERR_INVALID;
   }
-  GHB_CUDA_TRY(cudaMemcpy(out.d_group_perm[k], perm.data(), sizeof(int) * p.M, cudaMemcpyHostToDevice));
-  GHB_CUDA_TRY(cudaMemcpy(out.d_group_perm[k] + p.M, nat.data(), sizeof(int) * p.M, cudaMemcpyHostToDevice));
+  perm.insert(perm.end(), nat.begin(), nat.end());
+  GHB_CUDA_TRY(cudaMemcpy(out.d_group_perm[k], perm.data(), sizeof(int) * perm.size(), cudaMemcpyHostToDevice));
   GHB_CUDA_TRY(cudaStreamSynchronize(cudaStreamLegacy));   // in place before any stream's kernels read it
   (k == 0 ? p.fx : p.rt) = f;
   out.cap[k] = cap;
@@ -315,41 +316,45 @@ ghb_status make_plan_untuned(int M, PlanHolder& out) {
   ghb_status st = build_plan_tables(M, out.plan, t);
   if (st != GHB_OK) return st;
   FftPlan& p = out.plan;
-  const std::vector<float2>& tw32 = t.tw32;
-  for (int k = 0; k < 2; ++k) GHB_CUDA_TRY(cudaMalloc(&out.d_group_perm[k], sizeof(int) * 2 * M));
-  GHB_CUDA_TRY(cudaMalloc(&out.d_fx_tw, sizeof(fxw) * M));
-  GHB_CUDA_TRY(cudaMalloc(&out.d_tw32, sizeof(float2) * M));
+  // all tables in one block, copied at once (one allocation, copy and wait: an image
+  // context makes plans at every change of its image)
+  std::vector<char> h;
+  auto put = [&h](const auto& v) {
+    const size_t at = h.size();
+    h.resize((at + sizeof(v[0]) * v.size() + 255) & ~static_cast<size_t>(255));
+    std::memcpy(h.data() + at, v.data(), sizeof(v[0]) * v.size());
+    return at;
+  };
+  size_t group[2];
   for (int k = 0; k < 2; ++k) {
-    GHB_CUDA_TRY(cudaMemcpy(out.d_group_perm[k], t.perm_of[k].data(), sizeof(int) * M, cudaMemcpyHostToDevice));
-    GHB_CUDA_TRY(cudaMemcpy(out.d_group_perm[k] + M, t.nat_of[k].data(), sizeof(int) * M, cudaMemcpyHostToDevice));
+    std::vector<int> both = t.perm_of[k];
+    both.insert(both.end(), t.nat_of[k].begin(), t.nat_of[k].end());
+    group[k] = put(both);
   }
-  GHB_CUDA_TRY(cudaMemcpy(out.d_fx_tw, t.fx_tw.data(), sizeof(fxw) * M, cudaMemcpyHostToDevice));
-  GHB_CUDA_TRY(cudaMemcpy(out.d_tw32, tw32.data(), sizeof(float2) * M, cudaMemcpyHostToDevice));
-  GHB_CUDA_TRY(cudaStreamSynchronize(cudaStreamLegacy));   // pageable copies: in place before other streams read
-  if (ct_size(M) && ct_plan(M).ok) {
-    std::vector<int> pct(M);
-    ct_perm(M, pct.data());
-    GHB_CUDA_TRY(cudaMalloc(&out.d_perm_ct, sizeof(int) * M));
-    GHB_CUDA_TRY(cudaMemcpy(out.d_perm_ct, pct.data(), sizeof(int) * M, cudaMemcpyHostToDevice));
+  const size_t fx = put(t.fx_tw), tw = put(t.tw32);
+  const bool ct = ct_size(M) && ct_plan(M).ok;
+  std::vector<int> pct(ct ? M : 0);
+  if (ct) ct_perm(M, pct.data());
+  const size_t perm_ct = put(pct);
+  GHB_CUDA_TRY(cudaMalloc(&out.d_tables, h.size()));
+  GHB_CUDA_TRY(cudaMemcpy(out.d_tables, h.data(), h.size(), cudaMemcpyHostToDevice));
+  GHB_CUDA_TRY(cudaStreamSynchronize(cudaStreamLegacy));   // a pageable copy: in place before other streams read
+  for (int k = 0; k < 2; ++k) {
+    out.d_group_perm[k] = reinterpret_cast<int*>(out.d_tables + group[k]);
+    out.cap[k] = kGroupCap[k];
+    FxPlan& f = k == 0 ? p.fx : p.rt;
+    f.perm = out.d_group_perm[k];
+    f.nat = out.d_group_perm[k] + M;
   }
-  p.ct = CtTables{out.d_perm_ct, out.d_tw32};
-  p.ct_col = p.ct_row = (out.d_perm_ct != nullptr) ? 1 : 0;
-  p.fx.perm = out.d_group_perm[0];
-  p.rt.perm = out.d_group_perm[1];
-  p.fx.nat = out.d_group_perm[0] + M;
-  p.rt.nat = out.d_group_perm[1] + M;
-  p.fx.tw = out.d_fx_tw;
-  for (int k = 0; k < 2; ++k) out.cap[k] = kGroupCap[k];
-  p.rt.tw32 = out.d_tw32;
+  p.fx.tw = reinterpret_cast<const fxw*>(out.d_tables + fx);
+  p.rt.tw32 = reinterpret_cast<const float2*>(out.d_tables + tw);
+  p.ct = CtTables{ct ? reinterpret_cast<const int*>(out.d_tables + perm_ct) : nullptr, p.rt.tw32};
+  p.ct_col = p.ct_row = ct ? 1 : 0;
   return GHB_OK;
 }
 
 void free_plan(PlanHolder& p) {
-  if (p.d_perm_ct) cudaFree(p.d_perm_ct);
-  for (int* q : p.d_group_perm)
-    if (q) cudaFree(q);
-  if (p.d_fx_tw) cudaFree(p.d_fx_tw);
-  if (p.d_tw32) cudaFree(p.d_tw32);
+  if (p.d_tables) cudaFree(p.d_tables);
   p = PlanHolder{};
 }
 

@@ -236,7 +236,8 @@ ghb_status get_plan(ghb_batch* b, int M, const FftPlan** dpl, FftPlan* hpl) {
     PlanEntry e;
     TRYB(make_plan(M, e.h));
     GHB_CUDA_TRY(cudaMalloc(&e.d_plan, sizeof(FftPlan)));
-    GHB_CUDA_TRY(cudaMemcpy(e.d_plan, &e.h.plan, sizeof(FftPlan), cudaMemcpyHostToDevice));
+    // on the batch's stream: ahead of its kernels (a pageable source, staged before return)
+    GHB_CUDA_TRY(cudaMemcpyAsync(e.d_plan, &e.h.plan, sizeof(FftPlan), cudaMemcpyHostToDevice, b->stream));
     it = b->plans.emplace(M, e).first;
   }
   *dpl = it->second.d_plan;

@@ -128,7 +128,8 @@ FieldGeom fgeom_of(const Geometry& g) { return make_field_geom(g.d, g.N[0], g.N[
 // Work-item arrays of the launches of one phase: appended to a pinned host
 // buffer, copied to the device with one transfer (flush) before the launches
 // that read them, and reset only after a stream synchronisation (when no queued
-// kernel can still read them).
+// kernel can still read them).  The kernels look their item up ahead of grid_wait()
+// (launch_util.cuh), so nothing but such copies on the batch's stream may write items.
 struct Arena {
   char* h = nullptr;
   char* d = nullptr;

@@ -378,12 +378,15 @@ ghb_status ghb_gram_noalloc(int d, const int* N, const int* M, const double* gri
  *                  chosen at each launch from the operand's shape: the widest
  *                  tile that leaves room for three CTAs on an SM and makes two
  *                  for each; else 1, 2, 4, 8 or 16 within shared memory, forced)
- *   cfg[2] rows32  rows per CTA of the FP32 2-D last-axis pass (0 = size rule;
- *                  1 or 2: the least rows that fill complex lines, once or twice)
+ *   cfg[2] rows32  rows per CTA of the FP32 last-axis pass (0 = size rule; 1 or 2:
+ *                  the least rows that fill complex lines, one for d = 2 and two for
+ *                  d = 3, once or twice)
  *   cfg[3] ct_col  1: size-specialised FP32 column kernels (only for lengths
  *                  that have them: 72, 135, 162, 270, 486, 1458, 2187,
  *                  4374), 0: runtime plan
- *   cfg[4] ct_row  the same for the last-axis pass
+ *   cfg[4] ct_row  the same for the last-axis pass (the autotuner decides it for d =
+ *                  2 and d = 3 apart and reports d = 2; a value set holds for both,
+ *                  unless the whole configuration is the one it reported)
  *   cfg[5] cap64   as cap32 for FP64 (no pass larger than 10)
  *   cfg[6] tile64  as tile32 for FP64
  * The first plan for M in a process times the candidates for cfg[2], [3], [4]

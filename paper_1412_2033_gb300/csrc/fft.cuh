@@ -140,6 +140,7 @@ struct FftPlan {
   int tile[2];               // column-pass tile width ([0] FP64, [1] FP32)
   int rows32;                // rows per CTA of the FP32 2-D operator's last-axis pass
   int ct_col, ct_row;        // 1: size-specialised FP32 kernels for the column / last-axis passes
+  int ct_row3;               // the same for the last-axis pass of three components (d = 3)
 };
 
 template <typename T> struct CT;

@@ -234,7 +234,7 @@ ghb_status launch_row<float>(int mode, const RowArgs& a, const FftPlan& pl, cuda
   int rows_per_cta = 1, NL = 1;
   row_lines(mode, a.nfields, a.ncomp, pl.M, pl.rows32, &rows_per_cta, &NL);
   if (mode == ROW_MATVEC) {   // set-up and Gram passes run in FP64 only
-    if (use_ct(pl, pl.ct_row != 0)) return launch_row_ct(NL, a, pl, rows_per_cta, s);
+    if (use_ct(pl, (a.ncomp == 3 ? pl.ct_row3 : pl.ct_row) != 0)) return launch_row_ct(NL, a, pl, rows_per_cta, s);
     if (!row_admitted(pl.M, NL, sizeof(float2))) {
       set_error("row transform too large for one CTA: M=" + std::to_string(pl.M));
       return GHB_ERR_INVALID;

@@ -349,7 +349,7 @@ ghb_status make_plan_untuned(int M, PlanHolder& out) {
   p.fx.tw = reinterpret_cast<const fxw*>(out.d_tables + fx);
   p.rt.tw32 = reinterpret_cast<const float2*>(out.d_tables + tw);
   p.ct = CtTables{ct ? reinterpret_cast<const int*>(out.d_tables + perm_ct) : nullptr, p.rt.tw32};
-  p.ct_col = p.ct_row = ct ? 1 : 0;
+  p.ct_col = p.ct_row = p.ct_row3 = ct ? 1 : 0;
   return GHB_OK;
 }
 

@@ -7,7 +7,9 @@
 //                 largest passes of 16 are the best at every length measured);
 //   rows32        rows per CTA of the FP32 2-D operator's last-axis pass;
 //   ct_col/ct_row size-specialised FP32 kernels (where compiled) or the
-//                 run-time-plan ones.  Measured last-axis pass: M = 270 203 us
+//                 run-time-plan ones, the last-axis pass for d = 2 and d = 3
+//                 apart (M = 162: 14.6 us specialised against 11.8 at N = 81, 47.5
+//                 against 66 at N = 81 in d = 3).  Measured last-axis pass: M = 270 203 us
 //                 specialised against 295, M = 4374 145 against 208; columns at
 //                 M = 4374 64 + 60 against 82 + 74.
 // The columns per CTA of the column passes (tile32/64) depend on the operand,
@@ -25,6 +27,7 @@
 // process.
 // GHB_AUTOTUNE=0 in the environment keeps the size rules instead.
 #include <algorithm>
+#include <array>
 #include <cstdlib>
 #include <cstring>
 #include <map>
@@ -43,11 +46,16 @@ namespace {
 
 struct Tune {
   int cap32, tile32, rows32, ct_col, ct_row, cap64, tile64;
+  int ct_row3;   // ct_row of the d = 3 last-axis pass: timed apart, set with ct_row
 };
-constexpr int kTuneFields = 7;
+// the fields of ghb_tune_get and ghb_tune_set
+std::array<int, 7> fields(const Tune& t) {
+  return {t.cap32, t.tile32, t.rows32, t.ct_col, t.ct_row, t.cap64, t.tile64};
+}
 
 std::mutex g_mutex;
 std::map<int, Tune> g_tunes;
+std::map<int, Tune> g_tuned;   // what the tuner chose, for ghb_tune_set to recognise
 
 bool tuning_enabled() {
   const char* e = std::getenv("GHB_AUTOTUNE");
@@ -56,7 +64,7 @@ bool tuning_enabled() {
 
 Tune size_rules(int M) {
   const int ct = ct_size(M) ? 1 : 0;
-  return Tune{32, 0, 0, ct, ct, 18, 0};
+  return Tune{32, 0, 0, ct, ct, 18, 0, ct};
 }
 
 ghb_status write_tune(const Tune& t, PlanHolder& h) {
@@ -73,6 +81,7 @@ ghb_status write_tune(const Tune& t, PlanHolder& h) {
   const bool ct = p.ct.perm != nullptr && ct_size(p.M);
   p.ct_col = ct ? t.ct_col : 0;
   p.ct_row = ct ? t.ct_row : 0;
+  p.ct_row3 = ct ? t.ct_row3 : 0;
   return GHB_OK;
 }
 
@@ -251,6 +260,16 @@ ghb_status tune_length(int M, Tune* out) {
           best.rows32 = rows;
         }
       }
+      // d = 3: three lines a row pair, at two thirds of the rows in the same buffers
+      row.ncomp = 3;
+      row.rows = std::max<int64_t>(rows * 2 / 3, 1);
+      row.comp_stride = row.rows * h;
+      float t3[2];
+      for (int ct : {0, 1}) {
+        p.ct_row3 = ct;
+        TUNE_TRY(tm.time([&] { return launch_row<float>(ROW_MATVEC, row, p, tm.s); }, &t3[ct]));
+      }
+      best.ct_row3 = t3[1] < t3[0] ? 1 : 0;
     }
   }
   // FP64: grouping (the last-axis pass at one row per CTA)
@@ -307,6 +326,7 @@ ghb_status tune_of(int M, Tune* out) {
   if (tuning_enabled()) {
     const ghb_status st = tune_length(M, &t);
     if (st != GHB_OK) return st;
+    g_tuned[M] = t;
   }
   g_tunes[M] = t;
   *out = t;
@@ -337,8 +357,8 @@ ghb_status ghb_tune_get(int M, int* cfg) {
   Tune t{};
   const ghb_status st = tune_of(M, &t);
   if (st != GHB_OK) return st;
-  const int v[kTuneFields] = {t.cap32, t.tile32, t.rows32, t.ct_col, t.ct_row, t.cap64, t.tile64};
-  std::memcpy(cfg, v, sizeof(v));
+  const auto v = fields(t);
+  std::memcpy(cfg, v.data(), sizeof(v));
   return GHB_OK;
 }
 
@@ -348,13 +368,15 @@ ghb_status ghb_tune_set(int M, const int* cfg) {
     set_error("ghb_tune_set: M must factor into primes <= 31 and cfg must not be NULL");
     return GHB_ERR_INVALID;
   }
-  const Tune t{cfg[0], cfg[1], cfg[2], cfg[3], cfg[4], cfg[5], cfg[6]};
+  Tune t{cfg[0], cfg[1], cfg[2], cfg[3], cfg[4], cfg[5], cfg[6], cfg[4]};
   if (!valid_tune(M, t)) {
     set_error("ghb_tune_set: invalid configuration (caps 5..32, tiles 0/1/2/4/8/16 within shared memory, "
               "rows 0..2, specialised kernels 0/1 and only for lengths that have them)");
     return GHB_ERR_INVALID;
   }
   std::lock_guard<std::mutex> lock(g_mutex);
+  const auto it = g_tuned.find(M);
+  if (it != g_tuned.end() && fields(it->second) == fields(t)) t = it->second;   // the tuner's own, put back
   g_tunes[M] = t;
   return GHB_OK;
 }
@@ -363,6 +385,7 @@ ghb_status ghb_tune_reset(void) {
   clear_error();
   std::lock_guard<std::mutex> lock(g_mutex);
   g_tunes.clear();
+  g_tuned.clear();
   return GHB_OK;
 }
 

@@ -192,3 +192,30 @@ def test_forced_rows_are_launched(run):
       printf("%d %d", bad, n > 1000);
     """)
     assert out == ["0", "1"]
+
+
+def test_last_axis_choices_of_two_and_three_components(run):
+    """The autotuner times d = 2 and d = 3 last-axis passes apart: each takes the
+    size-specialised kernels by its own flag."""
+    out = run(r"""
+      FftPlan p{};
+      p.M = 162;
+      group_plan(1, 162, 32, p.rt, nullptr, nullptr, line_limit(1, 162, 1));
+      int some = 0;
+      p.ct.perm = &some;
+      for (int d : {2, 3})
+        for (int two : {0, 1})
+          for (int three : {0, 1}) {
+            RowArgs a{};
+            a.nfields = 1;
+            a.ncomp = d;
+            a.rows = 100000;
+            a.H = 41;
+            p.ct_row = two;
+            p.ct_row3 = three;
+            launched = 0;                       // run-time launches; the specialised ones are not counted
+            launch_row<float>(ROW_MATVEC, a, p, nullptr);
+            printf("%d", launched);
+          }
+    """)
+    assert out == ["11001010"]

@@ -35,9 +35,12 @@ inline ghb_status ensure_dyn_smem(F* func, int bytes, std::atomic<unsigned long 
 // behind it starts when it has completed and the later ones after that kernel, and
 // the next copy to the same place waits for every kernel queued before it.
 //
-// Measured, one operator application: N = 63 FP32 31.2 -> 19.1 us, N = 2187 273 ->
-// 262, N = 1023 79 -> 68, d = 3 N = 65 66 -> 53; FP64 N = 405 94 -> 83; bound pairs N =
-// 2187 146 -> 141 ms, d = 3 N = 65 174 -> 140 ms.  Letting the next grid in
+// Measured, the same kernels launched plainly and chained, one operator application
+// among others: N = 63 FP32 31.2 -> 19.1 us (20.2 now; plain launches of the passes before
+// the run-time plans 26.4), N = 2187 273 -> 262, N = 1023 79 -> 68, d = 3 N = 65 66 -> 53;
+// FP64 N = 405 94 -> 83; bound pairs N = 2187 146 -> 141 ms, d = 3 N = 65 174 -> 140 ms.
+// Where launches do not chain (ghb_profile records events between them) short passes
+// take longer than those did.  Letting the next grid in
 // earlier (griddepcontrol.launch_dependents after the wait) gives N = 63 18.6 us
 // but N = 2187 310 us and its bound pair 164 ms: blocks that only wait hold shared
 // memory and slots while the last blocks of the grid before still run.

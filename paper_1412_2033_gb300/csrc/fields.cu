@@ -468,7 +468,7 @@ __device__ void op_project(const CgItem& it, int64_t bid, int64_t nb) {
 }
 
 // x = 0, r = b, p = 0, <b, b>; the last block initialises the CG scalars.
-template <typename T>
+template <typename T, bool PAIR>
 __device__ void op_init(const CgItem& it, int64_t bid, int64_t nb) {
   using C = typename CT<T>::type;
   const FieldGeom& fg = it.fg;
@@ -477,7 +477,7 @@ __device__ void op_init(const CgItem& it, int64_t bid, int64_t nb) {
   C* p = static_cast<C*>(it.p);
   const C* b = static_cast<const C*>(it.b);
   CgState* st = it.st;
-  ThreadSum<T> acc;   // the cross-thread and cross-block sums in FP64
+  ThreadSum<T, PAIR> acc;   // the cross-thread and cross-block sums in FP64
   GHB_FIELD_LOOP(e, fg, bid, nb) {
     const int j = jindex(fg, e);
     const T wt = (j == 0) ? T(1) : T(2);
@@ -510,14 +510,14 @@ __device__ void op_init(const CgItem& it, int64_t bid, int64_t nb) {
 
 // Per-thread part of op_project_dot: q = G w on this thread's entries and
 // their share of <p, q>.
-template <typename T, int D>
+template <typename T, int D, bool PAIR>
 __device__ __forceinline__ double project_dot_loop(const CgItem& it, int64_t bid, int64_t nb) {
   using C = typename CT<T>::type;
   const FieldGeom& fg = it.fg;
   C* q = static_cast<C*>(it.q);
   const C* w = static_cast<const C*>(it.w);
   const C* p = static_cast<const C*>(it.p);
-  ThreadSum<T> acc;
+  ThreadSum<T, PAIR> acc;
   GHB_FIELD_LOOP(e, fg, bid, nb) {
     int k[3];
     int j;
@@ -543,12 +543,12 @@ __device__ __forceinline__ double project_dot_loop(const CgItem& it, int64_t bid
 }
 
 // q = G w, <p, q>; the last block forms alpha = <r, r> / <p, A p>.
-template <typename T>
+template <typename T, bool PAIR>
 __device__ void op_project_dot(const CgItem& it, int64_t bid, int64_t nb) {
   const FieldGeom& fg = it.fg;
   CgState* st = it.st;
   if (st->done != RUNNING) return;
-  const double acc = fg.d == 2 ? project_dot_loop<T, 2>(it, bid, nb) : project_dot_loop<T, 3>(it, bid, nb);
+  const double acc = fg.d == 2 ? project_dot_loop<T, 2, PAIR>(it, bid, nb) : project_dot_loop<T, 3, PAIR>(it, bid, nb);
   double tot;
   if (grid_sum_last(acc, it.partials, &st->ticket, &tot, bid, nb)) {
     st->pq = tot;
@@ -563,7 +563,7 @@ __device__ void op_project_dot(const CgItem& it, int64_t bid, int64_t nb) {
 
 // Per-thread part of op_update: x += alpha p, r -= alpha q on this thread's
 // entries and their share of <r, r>.
-template <typename T, int D>
+template <typename T, int D, bool PAIR>
 __device__ __forceinline__ double update_loop(const CgItem& it, T al, int64_t bid, int64_t nb) {
   using C = typename CT<T>::type;
   const FieldGeom& fg = it.fg;
@@ -571,7 +571,7 @@ __device__ __forceinline__ double update_loop(const CgItem& it, T al, int64_t bi
   C* r = static_cast<C*>(it.r);
   const C* p = static_cast<const C*>(it.p);
   const C* q = static_cast<const C*>(it.q);
-  ThreadSum<T> acc;
+  ThreadSum<T, PAIR> acc;
   GHB_FIELD_LOOP(e, fg, bid, nb) {
     const int j = jindex(fg, e);
     const T wt = (j == 0) ? T(1) : T(2);
@@ -600,13 +600,13 @@ __device__ __forceinline__ double update_loop(const CgItem& it, T al, int64_t bi
 }
 
 // x += alpha p, r -= alpha q, <r, r>; the last block forms beta and the stop test.
-template <typename T>
+template <typename T, bool PAIR>
 __device__ void op_update(const CgItem& it, int64_t bid, int64_t nb) {
   const FieldGeom& fg = it.fg;
   CgState* st = it.st;
   if (st->done != RUNNING) return;
   const T al = static_cast<T>(st->alpha);
-  const double acc = fg.d == 2 ? update_loop<T, 2>(it, al, bid, nb) : update_loop<T, 3>(it, al, bid, nb);
+  const double acc = fg.d == 2 ? update_loop<T, 2, PAIR>(it, al, bid, nb) : update_loop<T, 3, PAIR>(it, al, bid, nb);
   double tot;
   if (grid_sum_last(acc, it.partials, &st->ticket, &tot, bid, nb)) {
     const double rr_old = st->rr;
@@ -669,11 +669,11 @@ __device__ void op_accum(const CgItem& it, int64_t bid, int64_t nb) {
   }
 }
 
-template <typename T, int OP>
+template <typename T, int OP, bool PAIR>
 __device__ __forceinline__ void run_op(const CgItem& it, int64_t bid, int64_t nb) {
-  if constexpr (OP == CG_INIT) op_init<T>(it, bid, nb);
-  else if constexpr (OP == CG_PROJECT_DOT) op_project_dot<T>(it, bid, nb);
-  else if constexpr (OP == CG_UPDATE) op_update<T>(it, bid, nb);
+  if constexpr (OP == CG_INIT) op_init<T, PAIR>(it, bid, nb);
+  else if constexpr (OP == CG_PROJECT_DOT) op_project_dot<T, PAIR>(it, bid, nb);
+  else if constexpr (OP == CG_UPDATE) op_update<T, PAIR>(it, bid, nb);
   else if constexpr (OP == CG_PROJECT) op_project<T>(it, bid, nb);
   else if constexpr (OP == CG_RESIDUAL) op_residual(it, bid, nb);
   else if constexpr (OP == CG_TO_F32) op_to_f32(it, bid, nb);
@@ -683,7 +683,7 @@ __device__ __forceinline__ void run_op(const CgItem& it, int64_t bid, int64_t nb
 template <typename T, int OP>
 __global__ void __launch_bounds__(kFieldThreads) cg_kernel(CgItem it) {
   grid_wait();
-  run_op<T, OP>(it, blockIdx.x, gridDim.x);
+  run_op<T, OP, false>(it, blockIdx.x, gridDim.x);
 }
 
 template <typename T, int OP>
@@ -693,7 +693,7 @@ __global__ void __launch_bounds__(kFieldThreads) cg_kernel_batch(const CgItem* _
   __syncthreads();
   const CgItem& it = items[s_item];
   grid_wait();
-  run_op<T, OP>(it, blockIdx.x - it.block_begin, it.nblocks);
+  run_op<T, OP, true>(it, blockIdx.x - it.block_begin, it.nblocks);
 }
 
 __global__ void to_f32_real_kernel(float* dst, const double* src, int64_t n) {

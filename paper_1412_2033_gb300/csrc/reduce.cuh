@@ -5,11 +5,12 @@
 
 namespace ghb {
 
-// A thread's part of an inner product.  FP32: one entry's products are summed in FP32
-// and the entries in two floats, with the rounding of every sum kept (Knuth's
-// two-sum), so that a thread may take any number of entries and its sum is no coarser
-// than one entry's.  FP64: a plain sum.  An entry starts from open() and ends in close().
-template <typename T>
+// A thread's part of an inner product: a plain sum in the field's precision or, in the
+// batched kernels on FP32 fields (PAIR), one entry's products in FP32 and the entries in
+// two floats with the rounding of every sum kept (Knuth's two-sum), so that a thread
+// may take several entries where it took one and its sum is no coarser.  An entry
+// starts from open() and ends in close().
+template <typename T, bool PAIR>
 struct ThreadSum {
   T v = T(0);
   __host__ __device__ __forceinline__ T open() const { return v; }
@@ -17,7 +18,7 @@ struct ThreadSum {
   __host__ __device__ __forceinline__ double total() const { return v; }
 };
 template <>
-struct ThreadSum<float> {
+struct ThreadSum<float, true> {
   float v = 0.0f, low = 0.0f;
   __host__ __device__ __forceinline__ float open() const { return 0.0f; }
   __host__ __device__ __forceinline__ void close(float s) {
@@ -25,12 +26,7 @@ struct ThreadSum<float> {
     low += (v - (t - u)) + (s - u);
     v = t;
   }
-  // (one entry leaves low = 0: a warp of such threads skips two FP64 instructions, 1 % of
-  // a d = 3 N = 65 bound pair)
-  __host__ __device__ __forceinline__ double total() const {
-    const double s = static_cast<double>(v);
-    return low == 0.0f ? s : s + static_cast<double>(low);
-  }
+  __host__ __device__ __forceinline__ double total() const { return static_cast<double>(v) + static_cast<double>(low); }
 };
 
 template <typename T>

@@ -16,7 +16,7 @@ int main() {
   for (int n : {1, 2, 8, 16, 1000, 100000}) {
     double worst = 0;
     for (int repeat = 0; repeat < 20; ++repeat) {
-      ghb::ThreadSum<float> sum;
+      ghb::ThreadSum<float, true> sum;
       double exact = 0;
       for (int i = 0; i < n; ++i) {
         const float s = std::ldexp(u(rng), int(rng() % 12));   // entries of an inner product, of mixed size

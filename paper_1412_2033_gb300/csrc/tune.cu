@@ -262,6 +262,7 @@ ghb_status tune_length(int M, Tune* out) {
       }
       // d = 3: three lines a row pair, at two thirds of the rows in the same buffers
       row.ncomp = 3;
+      p.rows32 = best.rows32;
       row.rows = std::max<int64_t>(rows * 2 / 3, 1);
       row.comp_stride = row.rows * h;
       float t3[2];
